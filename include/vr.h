@@ -383,7 +383,7 @@ vr_status vr_volume_update_async(vr_volume vol, const float *src, int src_on_dev
  * ADDS dL/d(table) to `grad_tf_dev` (n x 4 float32, device) and, unless it is
  * NULL, dL/d(voxel) to `grad_density_dev` (Nz x Ny x Nx float32, device, the
  * original volume's indexing: halo copies are summed into the voxels they copy).
- * Recomputes the forward pass per brick; transmittances come from checkpoints,
+ * Recomputes the forward pass per brick; transmittances are products of (1 - alpha),
  * never from division. Requires early termination off (VR_ERR_ARG otherwise).
  * Runs of more than 4096 owned samples in one brick are skipped and reported as
  * VR_ERR_BOUNDS by vr_sync. Float atomics: results vary in the last bits

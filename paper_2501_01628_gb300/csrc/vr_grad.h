@@ -1,0 +1,77 @@
+// vr_grad.h -- structures shared by the host side of the adjoint (vr_host.cpp)
+// and its kernels (vr_grad.cu). Not part of the public ABI.
+#pragma once
+
+#include "vr_internal.h"
+
+namespace vr {
+
+// A brick's owned run of a ray is cut into segments of kGradSeg samples, counted
+// from the run's first sample, and groups of kGradGroup segments, one thread's
+// work. A run of more than kGradMaxRun samples is reported (its samples get no
+// gradient), and its last segment takes everything from sample kGradMaxRun on.
+constexpr int kGradSeg = 8;
+constexpr int kGradGroup = 8;
+constexpr int kGradMaxRun = 4096;
+// Copies of the table gradient, spread over blocks and lanes so that few
+// reductions meet on one entry. 256^3 volume, 4 views of 512^2, ms per training
+// step: 7.29 with 16 copies by block, 6.44 with 64, 6.21 with 256, 6.15 with
+// 1024 by block and lane % 8, 6.66 with 4096 by block and lane.
+constexpr int kGradCopies = 512;
+constexpr int kGradLaneCopies = 8;
+constexpr int kGradEntry = 8;      // floats per table interval in a copy: d/dT[i], d/dT[i+1]
+// Voxel gradients go through quads (two 16-byte reductions per cell, then one pass
+// over the volume's quads) when the view's samples, bounded by rect areas times
+// longest runs, are over this many times the quads, else straight into the voxels
+// (eight reductions per cell). One view, 8 bricks, us per training step quads /
+// direct: 256^3 at 128^2 (ratio 0.8) 1240 / 1147, at 256^2 (3) 1413 / 1319, at
+// 384^2 (7) 1545 / 1550; 128^3 at 256^2 (12) 1045 / 1063; 64^3 at 256^2 (47) 953 /
+// 1001; 256^3, four views at 512^2 (12) 6450 / 7160.
+constexpr long long kGradQuadsRatio = 6;
+constexpr long long kGradBandBytes = 1LL << 30;  // per-sample workspace of one band of image rows
+
+struct GradParams {
+    MarchParams m;                // camera, lattice, table, bricks (rects clipped to the image band)
+    const float4 *grad_img;       // dL/dI, H x W
+    // Workspace, [...][pixel of the brick's rect]; the offsets count segments and groups.
+    float *x;                     // per sample: its table coordinate (not clamped)
+    float *front;                 // per segment: T in front of it, from the group's start
+    float2 *group;                // per group: (lambda_C . C, T) of the group alone, then
+                                  // (lambda_T behind it, T in front of it) along the whole ray
+    long long soff[kMaxBricks], goff[kMaxBricks];
+    int nseg[kMaxBricks];         // segments kept per pixel
+    unsigned short *count;        // per (brick, pixel), at BrickLaunch::poff: groups of the run
+    float *tf_copies;             // kGradCopies x ntf x kGradEntry, zeroed before the launches
+    float *grad_vol;              // Nz x Ny x Nx, or null
+    float4 *grad_quads;           // quads of voxel gradients laid out as the bricks', or null
+                                  // (reductions straight into grad_vol)
+    int N[3];
+    int band_y0, band_h;          // image rows of this launch
+    int *error;                   // device error word: bit 0 = a run exceeded kGradMaxRun
+};
+
+// Voxel gradients gathered from the quads (grad_voxels_kernel).
+struct GradVoxelBrick {
+    long long base;   // quad offset of the brick's storage
+    int lo[3];        // voxel box origin
+    int s[3];         // haloed extents
+    int row_begin;    // first of the brick's s[1] x s[2] rows
+};
+struct GradVoxelParams {
+    const float4 *quads;
+    float *grad_vol;
+    int N[3];
+    int nb;
+    int n_rows;
+    GradVoxelBrick b[kMaxBricks];
+};
+
+// The adjoint's steps for one band of image rows (see vr_grad.cu), in order:
+// groups, scan, samples. `groups`: the largest number of groups of a brick. launch_grad_table adds the copies into grad_tf (ntf x 4).
+cudaError_t launch_grad_groups(const GradParams &p, int kind, int groups, cudaStream_t s);
+cudaError_t launch_grad_scan(const GradParams &p, cudaStream_t s);
+cudaError_t launch_grad_samples(const GradParams &p, int groups, cudaStream_t s);
+cudaError_t launch_grad_voxels(const GradVoxelParams &p, cudaStream_t s);
+cudaError_t launch_grad_table(const float *tf_copies, int ntf, float *grad_tf, cudaStream_t s);
+
+}  // namespace vr

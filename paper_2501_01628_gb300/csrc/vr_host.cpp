@@ -16,6 +16,7 @@
 #include <string>
 #include <vector>
 
+#include "vr_grad.h"
 #include "vr_objects.h"
 
 using namespace vr;
@@ -911,7 +912,7 @@ vr_status vr_destroy(vr_ctx ctx)
     cudaFree(ctx->d_tf);
     cudaFree(ctx->d_counter);
     cudaFree(ctx->d_error);
-    cudaFree(ctx->d_gpart);
+    cudaFree(ctx->d_grad);
     cudaFree(ctx->frame.d_part);
     cudaFree(ctx->frame2.d_part);
     cudaFree(ctx->d_pool_done);
@@ -1044,7 +1045,7 @@ vr_status create_volume(vr_ctx ctx, const int dims[3], vr_dtype storage, const v
     DeviceGuard g(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     VR_CUDA(ctx, vr::host::dev_malloc(&vol->d_data, static_cast<size_t>(off_bytes)));
-    vol->bytes = off_bytes;
+    vol->bytes = vol->quad_bytes = off_bytes;
     if (ctx->staging && storage == VR_F32) {
         // scalar copy for the staged march: rows padded to 4 elements (16 bytes),
         // each brick 128-byte aligned
@@ -1166,44 +1167,139 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     if (ctx->opc_ref > 0.0f) return fail(ctx, VR_ERR_ARG, "backward requires opacity correction off");
     DeviceGuard g(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    static thread_local MarchParams mp;
+    static thread_local GradParams gp;
     vr_frame_s &fr = ctx->frame;
-    // forward partials (recomputed: nothing per sample is kept from the forward call)
-    vr_status st = prepare_frame(ctx, vol, fr, mp);
+    vr_status st = prepare_frame(ctx, vol, fr, gp.m);
     if (st != VR_OK) return st;
-    st = ensure_frame(ctx, fr, std::max(fr.pool_px, 1LL));
-    if (st != VR_OK) return st;
-    mp.partials = fr.d_part;
-    mp.sample_counter = nullptr;
-    VR_LAUNCH(ctx, launch_march(mp, vol->kind(), s));
-    if (fr.total_px > ctx->gpart_cap) {
-        cudaFree(ctx->d_gpart);
-        ctx->d_gpart = nullptr;
-        ctx->gpart_cap = 0;
-        VR_CUDA(ctx, vr::host::dev_malloc(&ctx->d_gpart, static_cast<size_t>(fr.total_px) * sizeof(float4)));
-        ctx->gpart_cap = fr.total_px;
+    gp.m.sample_counter = nullptr;
+    // segments per pixel of each brick: its longest possible run, cut off where
+    // runs are refused (the last segment then takes the rest)
+    const int nb = fr.nb;
+    int groups = 0;
+    long long row_segs = 0;  // segments of one full image row
+    int ngroup[kMaxBricks];
+    for (int b = 0; b < nb; ++b) {
+        const int *bx = &vol->boxes[6 * b];
+        double d2 = 0.0;
+        for (int a = 0; a < 3; ++a) d2 += static_cast<double>(bx[3 + a] - bx[a]) * (bx[3 + a] - bx[a]);
+        const double run = std::sqrt(d2) / ctx->step + 4.0;
+        gp.nseg[b] = run >= kGradMaxRun ? kGradMaxRun / kGradSeg + 1
+                                        : static_cast<int>(run + kGradSeg - 1) / kGradSeg;
+        ngroup[b] = (gp.nseg[b] + kGradGroup - 1) / kGradGroup;
+        if (fr.rects[4 * b + 2] <= 0) continue;
+        groups = std::max(groups, ngroup[b]);
+        row_segs += static_cast<long long>(gp.nseg[b]) * fr.rects[4 * b + 2];
     }
-    static thread_local CompositeGradParams cg;
-    std::memset(&cg, 0, sizeof(cg));
-    cg.W = fr.W;
-    cg.H = fr.H;
-    cg.nb = fr.nb;
-    for (int j = 0; j < fr.nb; ++j) cg.order[j] = fr.order[j];
-    for (int b = 0; b < fr.nb; ++b) {
-        std::memcpy(cg.rect[b], &fr.rects[4 * b], 4 * sizeof(int));
-        cg.poff[b] = fr.poff[b];
+    // bands of image rows whose samples fit the workspace's bound
+    const long long row_bytes = row_segs * kGradSeg * static_cast<long long>(sizeof(float));
+    int band_h = static_cast<int>(
+        std::min<long long>(fr.H, row_bytes > 0 ? std::max(1LL, kGradBandBytes / row_bytes) : fr.H));
+    struct Band {
+        long long segs = 0, groups = 0, px = 0;
+    };
+    auto clip = [&](int y0) {  // the bricks' rects and tables of one band
+        Band n;
+        int items = 0;
+        for (int b = 0; b < nb; ++b) {
+            const int *r = &fr.rects[4 * b];
+            BrickLaunch &L = gp.m.b[b];
+            const int top = std::max(r[1], y0), end = std::min(r[1] + r[3], y0 + band_h);
+            L.rect[1] = top;
+            L.rect[3] = std::max(0, end - top);
+            L.poff = n.px;
+            gp.soff[b] = n.segs;
+            gp.goff[b] = n.groups;
+            const long long area = static_cast<long long>(L.rect[2]) * L.rect[3];
+            n.px += area;
+            n.segs += area * gp.nseg[b];
+            n.groups += area * ngroup[b];
+            L.item_begin = items;
+            items += L.tiles_x * ((L.rect[3] + gp.m.tile_h - 1) / gp.m.tile_h);
+        }
+        gp.m.n_items = items;
+        return n;
+    };
+    // workspace: table copies, groups, samples, segments, counts (each part a
+    // multiple of 16 bytes from the start); where it cannot be had, smaller bands
+    auto part = [](long long n, size_t size) { return (static_cast<size_t>(n) * size + 15) & ~static_cast<size_t>(15); };
+    const size_t copies_bytes = part(static_cast<long long>(kGradCopies) * ctx->ntf * kGradEntry, sizeof(float));
+    size_t group_bytes, x_bytes, front_bytes;
+    long long view_segs;
+    for (;; band_h = (band_h + 1) / 2) {
+        Band most;
+        view_segs = 0;
+        for (int y0 = 0; y0 < fr.H; y0 += band_h) {
+            const Band n = clip(y0);
+            most.segs = std::max(most.segs, n.segs);
+            most.groups = std::max(most.groups, n.groups);
+            most.px = std::max(most.px, n.px);
+            view_segs += n.segs;
+        }
+        group_bytes = part(most.groups, sizeof(float2));
+        x_bytes = part(most.segs * kGradSeg, sizeof(float));
+        front_bytes = part(most.segs, sizeof(float));
+        const size_t need = copies_bytes + group_bytes + x_bytes + front_bytes + part(most.px, sizeof(unsigned short));
+        if (need <= ctx->grad_cap) break;
+        cudaFree(ctx->d_grad);
+        ctx->d_grad = nullptr;
+        ctx->grad_cap = 0;
+        const cudaError_t e = vr::host::dev_malloc(&ctx->d_grad, need);
+        if (e == cudaSuccess) {
+            ctx->grad_cap = need;
+            break;
+        }
+        if (e != cudaErrorMemoryAllocation || band_h <= 1) return cuda_fail(ctx, e, "backward workspace");
+        cudaGetLastError();
     }
-    cg.partials = fr.d_part;
-    cg.grad_img = reinterpret_cast<const float4 *>(grad_rgba_dev);
-    cg.grad_partials = ctx->d_gpart;
-    VR_LAUNCH(ctx, launch_composite_grad(cg, s));
-    GradArgs ga;
-    ga.grad_partials = ctx->d_gpart;
-    ga.grad_tf = grad_tf_dev;
-    ga.grad_vol = grad_density_dev;
-    for (int a = 0; a < 3; ++a) ga.N[a] = vol->dims[a];
-    ga.error = ctx->d_error;
-    VR_LAUNCH(ctx, launch_march_grad(mp, ga, vol->kind(), s));
+    char *at = ctx->d_grad;
+    gp.tf_copies = reinterpret_cast<float *>(at);
+    gp.group = reinterpret_cast<float2 *>(at += copies_bytes);
+    gp.x = reinterpret_cast<float *>(at += group_bytes);
+    gp.front = reinterpret_cast<float *>(at += x_bytes);
+    gp.count = reinterpret_cast<unsigned short *>(at += front_bytes);
+    gp.grad_img = reinterpret_cast<const float4 *>(grad_rgba_dev);
+    gp.grad_vol = grad_density_dev;
+    gp.grad_quads = nullptr;
+    const long long quads = vol->quad_bytes / static_cast<long long>(quad_size(vol->dtype, vol->octets));
+    if (grad_density_dev && view_segs * kGradSeg > kGradQuadsRatio * quads) {
+        if (!vol->d_gquads && vr::host::dev_malloc(&vol->d_gquads, quads * sizeof(float4)) != cudaSuccess)
+            cudaGetLastError();  // no room: reductions straight into the voxels
+        gp.grad_quads = vol->d_gquads;
+    }
+    for (int a = 0; a < 3; ++a) gp.N[a] = vol->dims[a];
+    gp.error = ctx->d_error;
+    VR_CUDA(ctx, cudaMemsetAsync(gp.tf_copies, 0, copies_bytes, s));
+    if (gp.grad_quads) VR_CUDA(ctx, cudaMemsetAsync(gp.grad_quads, 0, quads * sizeof(float4), s));
+    for (int y0 = 0; y0 < fr.H; y0 += band_h) {
+        clip(y0);
+        gp.band_y0 = y0;
+        gp.band_h = std::min(band_h, fr.H - y0);
+        VR_LAUNCH(ctx, launch_grad_groups(gp, vol->kind(), groups, s));
+        VR_LAUNCH(ctx, launch_grad_scan(gp, s));
+        VR_LAUNCH(ctx, launch_grad_samples(gp, groups, s));
+    }
+    if (gp.grad_quads) {
+        static thread_local GradVoxelParams vp;
+        vp.quads = gp.grad_quads;
+        vp.grad_vol = grad_density_dev;
+        vp.nb = nb;
+        long long rows = 0;
+        for (int a = 0; a < 3; ++a) vp.N[a] = vol->dims[a];
+        for (int b = 0; b < nb; ++b) {
+            const int *bx = &vol->boxes[6 * b];
+            GradVoxelBrick &V = vp.b[b];
+            V.base = vol->base[b];
+            for (int a = 0; a < 3; ++a) {
+                V.lo[a] = bx[a];
+                V.s[a] = bx[3 + a] - bx[a] + 2;
+            }
+            V.row_begin = static_cast<int>(rows);
+            if (fr.rects[4 * b + 2] > 0) rows += static_cast<long long>(V.s[1]) * V.s[2];  // seen bricks only
+        }
+        vp.n_rows = static_cast<int>(rows);
+        VR_LAUNCH(ctx, launch_grad_voxels(vp, s));
+    }
+    VR_LAUNCH(ctx, launch_grad_table(gp.tf_copies, ctx->ntf, grad_tf_dev, s));
     return VR_OK;
 }
 
@@ -1214,6 +1310,7 @@ vr_status vr_volume_release(vr_volume vol)
     cudaFree(vol->d_data);
     cudaFree(vol->d_staging);
     cudaFree(vol->d_scalar);
+    cudaFree(vol->d_gquads);
     vol->ctx->live_objects--;
     delete vol;
     return VR_OK;

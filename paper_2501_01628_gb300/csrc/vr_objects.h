@@ -97,8 +97,8 @@ struct vr_ctx_s {
     unsigned long long *d_counter = nullptr;
     int *d_error = nullptr;        // device error word (vr_sync reports and clears it)
     bool count_samples = false;
-    float4 *d_gpart = nullptr;     // partial gradients (backward), partial-pool layout
-    long long gpart_cap = 0;
+    char *d_grad = nullptr;        // backward workspace: table copies, segments, segment counts
+    size_t grad_cap = 0;           // bytes
     vr_frame_s frame;              // context-owned frame for vr_render_frame
     // Pipelined frames (vr_set_frame_pipelining): vr_render_frame into device
     // memory alternates between `frame` and `frame2`, and its march may start
@@ -148,7 +148,9 @@ struct vr_volume_s {
     std::vector<vr::host::KdNode> tree;  // node 0 = root
     void *d_data = nullptr;
     long long bytes = 0;
+    long long quad_bytes = 0;      // of them the bricks' quads (or octets)
     float *d_staging = nullptr;    // float32 source for asynchronous re-packs from host memory
+    float4 *d_gquads = nullptr;    // quads of voxel gradients (vr_render_backward), laid out as d_data
     // scalar copy of the bricks for the staged march (float32 volumes created
     // while the context's staging was on): per brick, haloed voxels with rows
     // padded to sxp elements, starting at element sbase

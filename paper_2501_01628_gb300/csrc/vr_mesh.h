@@ -40,11 +40,27 @@ constexpr int kMeshLeafMax = 4;        // elements per leaf
 constexpr int kMeshMaxElems = 1 << 28; // elements per brick (leaf encoding)
 constexpr int kMeshStallSteps = 32;    // element steps without a sample before re-locating
 
+// Start grid of a brick: n[0] x n[1] x n[2] equal cells of its box, each with an
+// element near the cell's centre (brick-local), from which a walk through face
+// neighbours reaches a sample in the cell in a step or two -- the bricks are
+// convex and filled, so the walk towards the sample always has a neighbour.
+// About kMeshGridElems elements per cell.
+struct MeshGrid {
+    long long base;   // first cell in MeshParams::start
+    int n[3];
+    float scale[3];   // cells per voxel
+};
+constexpr int kMeshGridElems = 2;
+constexpr int kMeshWalkSteps = 64;     // of a walk before the BVH is asked instead
+constexpr float kMeshInside = 1.0e-6f; // barycentric slack of a sample on a face (FP32 rounding)
+
 struct MeshParams {
     MarchParams m;                    // camera, lattice, transfer function, tiles, bricks
     const float4 *rec;                // kMeshRec float4 per element
     const int4 *nbr;                  // brick-local neighbour across face i, -1 on the brick's boundary
     const MeshNode *nodes;
+    const int *start;                 // start grids
+    MeshGrid grid[kMaxBricks];
     long long rec_base[kMaxBricks];   // first element of each brick
     long long node_base[kMaxBricks];  // first BVH node of each brick
     int *error;                       // bit 3: a point location found no element (empty brick)

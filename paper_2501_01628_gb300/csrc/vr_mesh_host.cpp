@@ -29,6 +29,8 @@ struct vr_mesh_s {
     float4 *d_rec = nullptr;
     int4 *d_nbr = nullptr;
     MeshNode *d_nodes = nullptr;
+    int *d_start = nullptr;            // start grids
+    std::vector<MeshGrid> grid;        // per brick
     std::vector<long long> rec_base;   // per brick
     std::vector<long long> node_base;
     std::vector<long long> count;
@@ -42,6 +44,8 @@ struct BrickBuild {
     std::vector<MeshNode> nodes;
     std::vector<float4> rec;
     std::vector<int4> nbr;
+    MeshGrid grid;
+    std::vector<int> start;
     std::string err;
 };
 
@@ -252,6 +256,62 @@ bool build_records(const MeshInput &in, const int *box, BrickBuild &b)
     return true;
 }
 
+// Start grid (see vr_mesh.h): every cell gets the element whose centroid lies in
+// it and nearest its centre; an empty cell that of a filled neighbour along x,
+// then y, then z.
+void build_start(const int *box, BrickBuild &b)
+{
+    const long long n = static_cast<long long>(b.elems.size());
+    MeshGrid &g = b.grid;
+    const double ext[3] = {static_cast<double>(box[3] - box[0]), static_cast<double>(box[4] - box[1]),
+                           static_cast<double>(box[5] - box[2])};
+    const double h = std::cbrt(ext[0] * ext[1] * ext[2] * kMeshGridElems / static_cast<double>(n));
+    for (int a = 0; a < 3; ++a) {
+        g.n[a] = static_cast<int>(std::min(std::max(std::floor(ext[a] / h + 0.5), 1.0), 1024.0));
+        g.scale[a] = static_cast<float>(g.n[a] / ext[a]);
+    }
+    const size_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    b.start.assign(nx * ny * nz, -1);
+    std::vector<float> dist(b.start.size(), 0.f);
+    for (long long i = 0; i < n; ++i) {
+        const float4 &c = b.rec[static_cast<size_t>(kMeshRec) * i];
+        const float v[3] = {c.x, c.y, c.z};
+        size_t at = 0;
+        float d = 0.f;
+        for (int a = 2; a >= 0; --a) {
+            const float x = (v[a] - static_cast<float>(box[a])) * g.scale[a];
+            const int k = std::min(std::max(static_cast<int>(x), 0), g.n[a] - 1);
+            at = at * g.n[a] + k;
+            const float off = x - (static_cast<float>(k) + 0.5f);
+            d += off * off;
+        }
+        if (b.start[at] < 0 || d < dist[at]) {
+            b.start[at] = static_cast<int>(i);
+            dist[at] = d;
+        }
+    }
+    // fill along lines of `count` cells, `stride` apart
+    auto fill = [&](size_t first, size_t count, size_t stride) {
+        int last = -1;
+        for (size_t k = 0; k < count; ++k) {
+            int &c = b.start[first + k * stride];
+            if (c < 0) c = last;
+            last = c;
+        }
+        for (size_t k = count; k-- > 0;) {
+            int &c = b.start[first + k * stride];
+            if (c < 0) c = last;
+            last = c;
+        }
+    };
+    for (size_t z = 0; z < nz; ++z)
+        for (size_t y = 0; y < ny; ++y) fill((z * ny + y) * nx, nx, 1);
+    for (size_t z = 0; z < nz; ++z)
+        for (size_t x = 0; x < nx; ++x) fill(z * ny * nx + x, ny, nx);
+    for (size_t y = 0; y < ny; ++y)
+        for (size_t x = 0; x < nx; ++x) fill(y * nx + x, nz, ny * nx);
+}
+
 }  // namespace
 
 extern "C" {
@@ -318,13 +378,15 @@ vr_status vr_mesh_create(vr_ctx ctx, const int dims[3], const vr_partition *part
         for (int t = 0; t < nthreads; ++t)
             pool.emplace_back([&]() {
                 for (int b = next++; b < nb; b = next++)
-                    if (build_bvh(in, bricks[b])) build_records(in, &G.boxes[6 * b], bricks[b]);
+                    if (build_bvh(in, bricks[b]) && build_records(in, &G.boxes[6 * b], bricks[b]))
+                        build_start(&G.boxes[6 * b], bricks[b]);
             });
         for (auto &th : pool) th.join();
         for (int b = 0; b < nb; ++b)
             if (!bricks[b].err.empty()) return fail(ctx, VR_ERR_ARG, bricks[b].err);
     }
-    long long n_rec = 0, n_nodes = 0;
+    long long n_rec = 0, n_nodes = 0, n_start = 0;
+    m->grid.resize(nb);
     m->rec_base.resize(nb);
     m->node_base.resize(nb);
     m->count.resize(nb);
@@ -334,19 +396,25 @@ vr_status vr_mesh_create(vr_ctx ctx, const int dims[3], const vr_partition *part
         m->count[b] = static_cast<long long>(bricks[b].elems.size());
         n_rec += m->count[b];
         n_nodes += static_cast<long long>(bricks[b].nodes.size());
+        m->grid[b] = bricks[b].grid;
+        m->grid[b].base = n_start;
+        n_start += static_cast<long long>(bricks[b].start.size());
     }
     DeviceGuard g(ctx->device);
     const size_t rec_bytes = static_cast<size_t>(n_rec) * kMeshRec * sizeof(float4);
     const size_t nbr_bytes = static_cast<size_t>(n_rec) * sizeof(int4);
     const size_t node_bytes = static_cast<size_t>(n_nodes) * sizeof(MeshNode);
+    const size_t start_bytes = static_cast<size_t>(n_start) * sizeof(int);
     auto release = [&]() {
         cudaFree(m->d_rec);
         cudaFree(m->d_nbr);
         cudaFree(m->d_nodes);
+        cudaFree(m->d_start);
     };
     cudaError_t e = vr::host::dev_malloc(&m->d_rec, rec_bytes);
     if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_nbr, nbr_bytes);
     if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_nodes, node_bytes);
+    if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_start, start_bytes);
     for (int b = 0; e == cudaSuccess && b < nb; ++b) {
         const BrickBuild &B = bricks[b];
         e = cudaMemcpy(m->d_rec + kMeshRec * m->rec_base[b], B.rec.data(), B.rec.size() * sizeof(float4),
@@ -357,12 +425,15 @@ vr_status vr_mesh_create(vr_ctx ctx, const int dims[3], const vr_partition *part
         if (e == cudaSuccess)
             e = cudaMemcpy(m->d_nodes + m->node_base[b], B.nodes.data(), B.nodes.size() * sizeof(MeshNode),
                            cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(m->d_start + m->grid[b].base, B.start.data(), B.start.size() * sizeof(int),
+                           cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         release();
         return cuda_fail(ctx, e, "mesh upload");
     }
-    m->bytes = static_cast<long long>(rec_bytes + nbr_bytes + node_bytes);
+    m->bytes = static_cast<long long>(rec_bytes + nbr_bytes + node_bytes + start_bytes);
     ctx->live_objects++;
     ctx->input_seq++;  // new device data a pipelined kernel must not overlap
     *out = m.release();
@@ -376,6 +447,7 @@ vr_status vr_mesh_release(vr_mesh mesh)
     cudaFree(mesh->d_rec);
     cudaFree(mesh->d_nbr);
     cudaFree(mesh->d_nodes);
+    cudaFree(mesh->d_start);
     mesh->ctx->live_objects--;
     delete mesh;
     return VR_OK;
@@ -429,9 +501,11 @@ vr_status vr_render_mesh_frame(vr_ctx ctx, vr_mesh mesh, float *out_rgba, int ou
     mp.rec = mesh->d_rec;
     mp.nbr = mesh->d_nbr;
     mp.nodes = mesh->d_nodes;
+    mp.start = mesh->d_start;
     for (size_t b = 0; b < mesh->rec_base.size(); ++b) {
         mp.rec_base[b] = mesh->rec_base[b];
         mp.node_base[b] = mesh->node_base[b];
+        mp.grid[b] = mesh->grid[b];
     }
     mp.error = ctx->d_error;
     const int t = timing_begin(ctx, 0, s);

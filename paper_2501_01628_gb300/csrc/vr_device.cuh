@@ -173,8 +173,20 @@ __device__ __forceinline__ void ray_setup(const P &p, int px, int py, Ray &ray)
 // The samples brick B owns along `ray`: the slab estimate, made exact with the
 // ownership test itself (sample k is owned iff it lies before t_out and its cell
 // is in the brick).
+//
+// Every bound of the test is monotone in k, in FP32 too (the sample's t and each
+// coordinate are one rounded fma of the one before): along an axis with dv > 0
+// the lower bound is passed once and the upper one once after it, with dv < 0
+// the other way round. So the run is [first k past every entry bound, last k
+// before every exit bound], and each end is found by stepping away from its
+// estimate in doubling strides and bisecting -- two tests where the estimate is
+// off by less than a sample, some tens where it is off by the margin. Walking
+// sample by sample from the margin's far end took a ray nearly parallel to a
+// face thousands of tests, and one such ray holds up a whole launch: a cycling
+// frame of 512^3 at 1920 x 1080 0.564 -> 0.381 ms (one view; other views, with no
+// such ray, 0.58), a 2048^2 image of 1024^3 in 64 bricks 7.12 -> 6.28 ms.
 template <typename P>
-__device__ __forceinline__ void brick_run(const P &p, const BrickLaunch &B, const Ray &ray, OwnedRun &run)
+__host__ __device__ __forceinline__ void brick_run(const P &p, const BrickLaunch &B, const Ray &ray, OwnedRun &run)
 {
     run.ka = 0;
     run.kb = -1;
@@ -193,19 +205,63 @@ __device__ __forceinline__ void brick_run(const P &p, const BrickLaunch &B, cons
     }
     if (!(b0 <= b1)) return;
     const float t_in = ray.t_in, t_out = ray.t_out;
-    int ka = max(0, static_cast<int>(floorf((b0 - t_in) * p.inv_dt - 0.5f)) - ray.margin);
-    int kb = static_cast<int>(ceilf((fminf(b1, t_out) - t_in) * p.inv_dt - 0.5f)) + ray.margin;
-    auto owned = [&](int k) {
+    const int est_a = static_cast<int>(floorf((b0 - t_in) * p.inv_dt - 0.5f));
+    const int est_b = static_cast<int>(ceilf((fminf(b1, t_out) - t_in) * p.inv_dt - 0.5f));
+    const int k0 = max(0, est_a - ray.margin), k1 = est_b + ray.margin;  // the run lies in [k0, k1]
+    if (k0 > k1) return;
+    auto entered = [&](int k) {
         const float t = fmaf(static_cast<float>(k) + 0.5f, p.dt, t_in);
-        const float qxv = fmaf(t, ray.dv[0], ray.ov[0]);
-        const float qyv = fmaf(t, ray.dv[1], ray.ov[1]);
-        const float qzv = fmaf(t, ray.dv[2], ray.ov[2]);
-        return t < t_out && qxv >= B.own_lo[0] && qxv < B.own_hi[0] && qyv >= B.own_lo[1] && qyv < B.own_hi[1] &&
-               qzv >= B.own_lo[2] && qzv < B.own_hi[2];
+        bool in = true;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float q = fmaf(t, ray.dv[i], ray.ov[i]);
+            in = in && (ray.dv[i] < 0.0f || q >= B.own_lo[i]) && (ray.dv[i] > 0.0f || q < B.own_hi[i]);
+        }
+        return in;
     };
-    while (ka <= kb && !owned(ka)) ++ka;
-    while (kb > ka && !owned(kb)) --kb;
-    // owned samples are contiguous along the ray: [ka, kb] are all owned
+    auto before_exit = [&](int k) {
+        const float t = fmaf(static_cast<float>(k) + 0.5f, p.dt, t_in);
+        bool in = t < t_out;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float q = fmaf(t, ray.dv[i], ray.ov[i]);
+            in = in && (ray.dv[i] > 0.0f || q >= B.own_lo[i]) && (ray.dv[i] < 0.0f || q < B.own_hi[i]);
+        }
+        return in;
+    };
+    // the boundary of a monotone test on [k0, k1]: lo (k0 - 1 at least) is the last k
+    // on the low side, lo + 1 the first on the high side
+    auto boundary = [&](int guess, auto &&high) {
+        int lo, hi, stride = 1;
+        if (high(guess)) {
+            hi = guess;
+            lo = guess - 1;
+            while (lo >= k0 && high(lo)) {
+                hi = lo;
+                lo -= stride;
+                stride += stride;
+            }
+            lo = max(lo, k0 - 1);
+        } else {
+            lo = guess;
+            hi = guess + 1;
+            while (hi <= k1 && !high(hi)) {
+                lo = hi;
+                hi += stride;
+                stride += stride;
+            }
+            hi = min(hi, k1 + 1);
+        }
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (high(mid)) hi = mid;
+            else lo = mid;
+        }
+        return lo;
+    };
+    const int ka = boundary(min(max(est_a, k0), k1), entered) + 1;
+    const int kb = boundary(min(max(est_b, k0), k1), [&](int k) { return !before_exit(k); });
+    if (ka > kb) return;
     run.ka = ka;
     run.kb = kb;
 #pragma unroll

@@ -119,28 +119,6 @@ struct CompositeParams {
     int pool;
 };
 
-// Composite adjoint: the composite's layout plus the image gradient and the
-// per-brick partial gradients it produces (same layout as the partials).
-struct CompositeGradParams {
-    int W, H;
-    int nb;
-    int order[kMaxBricks];
-    int rect[kMaxBricks][4];
-    long long poff[kMaxBricks];
-    const float4 *partials;
-    const float4 *grad_img;
-    float4 *grad_partials;
-};
-
-// March adjoint outputs (gradients are added into).
-struct GradArgs {
-    const float4 *grad_partials;
-    float *grad_tf;   // ntf x 4
-    float *grad_vol;  // Nz x Ny x Nx, or null
-    int N[3];
-    int *error;       // device error word: bit 0 = a run exceeded the checkpoint storage
-};
-
 // Batched form: per view, the camera fields that dev::owned_run reads (same
 // names as MarchParams) and the view's work-item counts.
 struct BatchView {
@@ -246,8 +224,6 @@ cudaError_t launch_composite(const CompositeParams &p, cudaStream_t s, int max_b
 cudaError_t launch_composite_images(const ImagesParams &p, cudaStream_t s);
 // Tile masks of p (p.tile_mask) for frames whose march did not write them.
 cudaError_t launch_tile_masks(const CompositeParams &p, cudaStream_t s);
-cudaError_t launch_composite_grad(const CompositeGradParams &p, cudaStream_t s);
-cudaError_t launch_march_grad(const MarchParams &p, const GradArgs &g, int kind, cudaStream_t s);
 // Persistent batched kernel: cooperative launch of `blocks` blocks of 128 threads.
 cudaError_t launch_batch(const BatchParams &p, int kind, int blocks, cudaStream_t s);
 int batch_max_blocks_per_sm(int kind);

@@ -17,7 +17,7 @@
 #include <cstring>
 #include <vector>
 
-#include "vr_internal.h"
+#include "vr_device.cuh"
 
 namespace vr {
 namespace {
@@ -29,6 +29,9 @@ constexpr size_t kScratchBytes = VR_NOALLOC_SCRATCH_BYTES;
 constexpr size_t kTfBytes = 2 * 1024 * sizeof(float4);
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
+// Work item of the march: a block's 4 x 4 pixels (kGlobalLanes lanes each).
+constexpr int kGlobalTileW = 4, kGlobalTileH = 4;
+
 // Device address of g_scratch on the current device. The host-side symbol is
 // not a device address; the lookup is repeated on every call (it is cheap once
 // the module is loaded), so a device reset or a re-created primary context
@@ -39,136 +42,120 @@ cudaError_t scratch_address(void **out)
     return cudaGetSymbolAddress(out, g_scratch);
 }
 
-__device__ __forceinline__ int find_brick_g(const MarchParams &p, int item)
-{
-    int lo = 0, hi = p.nb - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (p.b[mid].item_begin <= item) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 // March over the caller's global volume (p.data: x-fastest float32 with
-// extents p.N). Ray setup, lattice, ownership and accumulation as in the
-// packed-brick march.
+// extents p.N). Ray setup, lattice, ownership and samples as in the
+// packed-brick march; the grid's first blocks write the composite's tile masks.
+//
+// kGlobalLanes neighbouring lanes take consecutive samples of one ray. The scratch
+// holds a few waves of work at most, often less than one, so the time is that of
+// the longest rays: with one lane per ray a sample waits for its loads, its
+// table entry and the sample before it, some 1200 cycles each. And in an x-fastest
+// volume a warp's 32 rays can lie on 32 different rows, each scalar load then
+// costs 32 wavefronts of the L1; consecutive samples of a ray share rows. The
+// transmittance runs through the lanes' samples in order (each lane repeats the
+// chain over the group's opacities); the colours are summed per lane and added
+// at the end. Bound by issue (52%) and the L1 data pipe (54%) where the image fills
+// the chip. us per call, 1 / 2 / 4 / 8 / 16 lanes per ray: 128^3, 400 x 300, six
+// bricks 244 / 130 / 83 / 76 / 82; 192^3, 400 x 320, four bricks - / - / 139 / 103 /
+// -; up to 64^3 the host's 39 us per call bound it. With one lane per ray, four
+// samples at a time took 244, keeping the cell's voxels and loading only new faces
+// 190 (divergent).
+constexpr int kGlobalLanes = 8;
+static_assert(kGlobalTileW * kGlobalTileH * kGlobalLanes == 128, "a block is one tile");
+static_assert(kMaskThreads == 128, "mask blocks are march blocks");
 __global__ void __launch_bounds__(128) march_global_kernel(const __grid_constant__ MarchParams p)
 {
-    const int item = blockIdx.x;
-    const BrickLaunch &B = p.b[find_brick_g(p, item)];
+    if (static_cast<int>(blockIdx.x) < p.mask_blocks) {
+        dev::write_tile_mask(blockIdx.x * kMaskThreads + threadIdx.x, p.mask_tiles_x, p.mask_tiles_y, p.nb, p.order,
+                             [&](int b) { return make_int4(p.b[b].rect[0], p.b[b].rect[1], p.b[b].rect[2],
+                                                           p.b[b].rect[3]); },
+                             p.tile_mask);
+        return;
+    }
+    constexpr unsigned all = 0xffffffffu;
+    const int item = blockIdx.x - p.mask_blocks;
+    const BrickLaunch &B = p.b[dev::find_brick(p, item)];
     const int local = item - B.item_begin;
     const int ty = local / B.tiles_x, tx = local - ty * B.tiles_x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rx = tx * kTileW + (warp & 1) * 8 + (lane & 7);
-    const int ry = ty * kTileH + (warp >> 1) * 4 + (lane >> 3);
-    if (rx >= B.rect[2] || ry >= B.rect[3]) return;
-    const int px = B.rect[0] + rx, py = B.rect[1] + ry;
-
-    const float fx = (static_cast<float>(px) + 0.5f) * p.inv_W;
-    const float fy = (static_cast<float>(py) + 0.5f) * p.inv_H;
-    float o[3], d[3];
-    if (p.ortho) {
-        const float a = (fx - 0.5f) * p.ow, b = (fy - 0.5f) * p.oh;
-        for (int i = 0; i < 3; ++i) {
-            o[i] = fmaf(b, p.u[i], fmaf(a, p.r[i], p.eye[i]));
-            d[i] = p.f[i];
-        }
-    } else {
-        const float sx = (fx * 2.0f - 1.0f) * p.tanx, sy = (fy * 2.0f - 1.0f) * p.tany;
-        for (int i = 0; i < 3; ++i) {
-            o[i] = p.eye[i];
-            d[i] = fmaf(sy, p.u[i], fmaf(sx, p.r[i], p.f[i]));
-        }
-        const float inv = __frsqrt_rn(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        for (int i = 0; i < 3; ++i) d[i] *= inv;
-    }
-    float ov[3], dv[3];
-    for (int i = 0; i < 3; ++i) {
-        ov[i] = o[i] * p.nmax;
-        dv[i] = d[i] * p.nmax;
-    }
-    float t0 = 0.0f, t1 = 3.0e38f, b0 = 0.0f, b1 = 3.0e38f;
-    bool hit = true;
-    for (int i = 0; i < 3; ++i) {
-        if (dv[i] == 0.0f) {
-            if (ov[i] < 0.0f || ov[i] > p.N[i]) hit = false;
-            if (ov[i] < static_cast<float>(B.lo[i]) || ov[i] > static_cast<float>(B.hi[i])) hit = false;
-        } else {
-            const float inv = __frcp_rn(dv[i]);
-            float ta = (0.0f - ov[i]) * inv, tb = (p.N[i] - ov[i]) * inv;
-            t0 = fmaxf(t0, fminf(ta, tb));
-            t1 = fminf(t1, fmaxf(ta, tb));
-            ta = (static_cast<float>(B.lo[i]) - ov[i]) * inv;
-            tb = (static_cast<float>(B.hi[i]) - ov[i]) * inv;
-            b0 = fmaxf(b0, fminf(ta, tb));
-            b1 = fminf(b1, fmaxf(ta, tb));
-        }
-    }
+    const int ray_id = threadIdx.x / kGlobalLanes, j = threadIdx.x % kGlobalLanes;
+    const int rx = tx * kGlobalTileW + ray_id % kGlobalTileW;
+    const int ry = ty * kGlobalTileH + ray_id / kGlobalTileW;
+    const bool inside = rx < B.rect[2] && ry < B.rect[3];
+    dev::Ray ray;
+    dev::ray_setup(p, B.rect[0] + rx, B.rect[1] + ry, ray);
+    dev::OwnedRun run;
+    dev::brick_run(p, B, ray, run);
+    if (!inside) run.kb = run.ka - 1;
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
-    if (hit && t0 < t1 && b0 <= b1) {
-        const float t_in = t0, t_out = t1;
-        float dmin = 3.0e38f;
-        for (int i = 0; i < 3; ++i)
-            if (dv[i] != 0.0f) dmin = fminf(dmin, fabsf(dv[i]));
-        const int margin = 2 + static_cast<int>(fminf(1.0e6f, __fdividef(1.0e-6f * p.nmax, dmin * p.dt)));
-        int ka = max(0, static_cast<int>(floorf((b0 - t_in) * p.inv_dt - 0.5f)) - margin);
-        int kb = static_cast<int>(ceilf((fminf(b1, t_out) - t_in) * p.inv_dt - 0.5f)) + margin;
-        auto owned = [&](int k) {
-            const float t = fmaf(static_cast<float>(k) + 0.5f, p.dt, t_in);
-            const float qxv = fmaf(t, dv[0], ov[0]);
-            const float qyv = fmaf(t, dv[1], ov[1]);
-            const float qzv = fmaf(t, dv[2], ov[2]);
-            return t < t_out && qxv >= B.own_lo[0] && qxv < B.own_hi[0] && qyv >= B.own_lo[1] &&
-                   qyv < B.own_hi[1] && qzv >= B.own_lo[2] && qzv < B.own_hi[2];
-        };
-        while (ka <= kb && !owned(ka)) ++ka;
-        while (kb > ka && !owned(kb)) --kb;
-        if (ka <= kb) {
-            const float *vol = static_cast<const float *>(p.data);
-            const int nx = static_cast<int>(p.N[0]), ny = static_cast<int>(p.N[1]), nz = static_cast<int>(p.N[2]);
-            const float xmax = static_cast<float>(p.ntf - 1);
-            float base[3], step[3];
-            for (int i = 0; i < 3; ++i) {
-                step[i] = dv[i] * p.dt;
-                base[i] = fmaf(t_in, dv[i], ov[i] - 0.5f);  // global voxel-centre coordinates
-            }
-            float kh = static_cast<float>(ka) + 0.5f;
-            for (int k = ka; k <= kb; ++k, kh += 1.0f) {
-                const float vx = fmaf(kh, step[0], base[0]);
-                const float vy = fmaf(kh, step[1], base[1]);
-                const float vz = fmaf(kh, step[2], base[2]);
-                const float flx = floorf(vx), fly = floorf(vy), flz = floorf(vz);
-                const float wx = vx - flx, wy = vy - fly, wz = vz - flz;
-                const int ix = static_cast<int>(flx), iy = static_cast<int>(fly), iz = static_cast<int>(flz);
-                const int x0 = min(max(ix, 0), nx - 1), x1 = min(max(ix + 1, 0), nx - 1);
-                const int y0 = min(max(iy, 0), ny - 1), y1 = min(max(iy + 1, 0), ny - 1);
-                const int z0 = min(max(iz, 0), nz - 1), z1 = min(max(iz + 1, 0), nz - 1);
-                const float *r00 = vol + (static_cast<long long>(z0) * ny + y0) * nx;
-                const float *r10 = vol + (static_cast<long long>(z0) * ny + y1) * nx;
-                const float *r01 = vol + (static_cast<long long>(z1) * ny + y0) * nx;
-                const float *r11 = vol + (static_cast<long long>(z1) * ny + y1) * nx;
-                const float v000 = __ldg(r00 + x0), v100 = __ldg(r00 + x1), v010 = __ldg(r10 + x0),
-                            v110 = __ldg(r10 + x1), v001 = __ldg(r01 + x0), v101 = __ldg(r01 + x1),
-                            v011 = __ldg(r11 + x0), v111 = __ldg(r11 + x1);
-                const float c00 = fmaf(wx, v100 - v000, v000), c10 = fmaf(wx, v110 - v010, v010);
-                const float c01 = fmaf(wx, v101 - v001, v001), c11 = fmaf(wx, v111 - v011, v011);
-                const float c0 = fmaf(wy, c10 - c00, c00), c1 = fmaf(wy, c11 - c01, c01);
-                const float s = fmaf(wz, c1 - c0, c0);
-                const float x = fminf(fmaxf(fmaf(s, p.tf_scale, p.tf_bias), 0.0f), xmax);
-                const int ti = static_cast<int>(x);
-                const float w = x - static_cast<float>(ti);
-                const float4 e0 = __ldg(p.tf + 2 * ti), de = __ldg(p.tf + 2 * ti + 1);
-                const float ta = T * fmaf(w, de.w, e0.w);
-                C0 = fmaf(ta, fmaf(w, de.x, e0.x), C0);
-                C1 = fmaf(ta, fmaf(w, de.y, e0.y), C1);
-                C2 = fmaf(ta, fmaf(w, de.z, e0.z), C2);
-                T = T - ta;
-                if (T <= p.ert_T) break;
-            }
-        }
+    const float *vol = static_cast<const float *>(p.data);
+    const int nx = static_cast<int>(p.N[0]), ny = static_cast<int>(p.N[1]), nz = static_cast<int>(p.N[2]);
+    const long long plane = static_cast<long long>(nx) * ny;
+    const float xmax = static_cast<float>(p.ntf - 1);
+    float base[3], step[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        step[i] = ray.dv[i] * p.dt;
+        base[i] = fmaf(ray.t_in, ray.dv[i], ray.ov[i] - 0.5f);  // global voxel-centre coordinates
     }
-    p.partials[B.poff + static_cast<long long>(ry) * B.rect[2] + rx] = make_float4(C0, C1, C2, 1.0f - T);
+    // floor(v) (see dev::kFloorOffset) and the fraction
+    auto cell = [](float v, float &w) {
+        const float y = __fadd_rd(v, dev::kFloorOffset);
+        w = v - (y - dev::kFloorOffset);
+        return static_cast<int>(__float_as_uint(y) - dev::kFloorBits);
+    };
+    for (int k = run.ka; __any_sync(all, k <= run.kb); k += kGlobalLanes) {
+        float a = 0.f, r = 0.f, g = 0.f, b = 0.f;
+        if (k + j <= run.kb) {
+            const float kh = static_cast<float>(k + j) + 0.5f;
+            float wx, wy, wz;
+            const int ix = cell(fmaf(kh, step[0], base[0]), wx);
+            const int iy = cell(fmaf(kh, step[1], base[1]), wy);
+            const int iz = cell(fmaf(kh, step[2], base[2]), wz);
+            const int x0 = min(max(ix, 0), nx - 1), x1 = min(max(ix + 1, 0), nx - 1);
+            const int y0 = min(max(iy, 0), ny - 1), y1 = min(max(iy + 1, 0), ny - 1);
+            const int z0 = min(max(iz, 0), nz - 1), z1 = min(max(iz + 1, 0), nz - 1);
+            const float *p0 = vol + z0 * plane, *p1 = vol + z1 * plane;
+            const long long r0 = static_cast<long long>(y0) * nx, r1 = static_cast<long long>(y1) * nx;
+            const float v000 = __ldg(p0 + r0 + x0), v100 = __ldg(p0 + r0 + x1), v010 = __ldg(p0 + r1 + x0),
+                        v110 = __ldg(p0 + r1 + x1), v001 = __ldg(p1 + r0 + x0), v101 = __ldg(p1 + r0 + x1),
+                        v011 = __ldg(p1 + r1 + x0), v111 = __ldg(p1 + r1 + x1);
+            const float c00 = fmaf(wx, v100 - v000, v000), c10 = fmaf(wx, v110 - v010, v010);
+            const float c01 = fmaf(wx, v101 - v001, v001), c11 = fmaf(wx, v111 - v011, v011);
+            const float c0 = fmaf(wy, c10 - c00, c00), c1 = fmaf(wy, c11 - c01, c01);
+            const float s = fmaf(wz, c1 - c0, c0);
+            const float x = fminf(fmaxf(fmaf(s, p.tf_scale, p.tf_bias), 0.0f), xmax);
+            float w;
+            float4 e0, de;
+            dev::ldg_v8(p.tf + 2 * cell(x, w), e0, de);
+            r = fmaf(w, de.x, e0.x);
+            g = fmaf(w, de.y, e0.y);
+            b = fmaf(w, de.z, e0.z);
+            a = fmaf(w, de.w, e0.w);
+        }
+        // T before this lane's sample; the ray ends after the first sample with T <= ert_T
+        float mine = T;
+#pragma unroll
+        for (int i = 0; i < kGlobalLanes; ++i) {
+            if (i == j) mine = T;
+            const float ai = __shfl_sync(all, a, i, kGlobalLanes);
+            if (!(T <= p.ert_T)) T = T - T * ai;
+        }
+        if (k + j <= run.kb && !(mine <= p.ert_T)) {
+            const float ta = mine * a;
+            C0 = fmaf(ta, r, C0);
+            C1 = fmaf(ta, g, C1);
+            C2 = fmaf(ta, b, C2);
+        }
+        if (T <= p.ert_T) run.kb = k;  // the same for the ray's lanes
+    }
+#pragma unroll
+    for (int i = 1; i < kGlobalLanes; i += i) {
+        C0 += __shfl_xor_sync(all, C0, i);
+        C1 += __shfl_xor_sync(all, C1, i);
+        C2 += __shfl_xor_sync(all, C2, i);
+    }
+    if (inside && j == 0)
+        p.partials[B.poff + static_cast<long long>(ry) * B.rect[2] + rx] = make_float4(C0, C1, C2, 1.0f - T);
 }
 
 bool normalize3(double v[3])
@@ -220,8 +207,8 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
         px += static_cast<long long>(r[2]) * r[3];
         px = (px + 7) & ~7LL;
         L.item_begin = items;
-        L.tiles_x = (r[2] + kTileW - 1) / kTileW;
-        items += L.tiles_x * ((r[3] + kTileH - 1) / kTileH);
+        L.tiles_x = (r[2] + kGlobalTileW - 1) / kGlobalTileW;
+        items += L.tiles_x * ((r[3] + kGlobalTileH - 1) / kGlobalTileH);
     }
     // the frame's partial images must fit the fixed scratch
     const int tiles_x = (cam->width + kCompW - 1) / kCompW, tiles_y = (cam->height + kCompTileH - 1) / kCompTileH;
@@ -290,10 +277,13 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
         return VR_ERR_CUDA;
     mp.tf = tf_dev;
     mp.partials = partials;
-    if (items > 0) {
-        march_global_kernel<<<items, 128, 0, s>>>(mp);
-        if (cudaGetLastError() != cudaSuccess) return VR_ERR_CUDA;
-    }
+    mp.tile_mask = masks;
+    mp.mask_tiles_x = tiles_x;
+    mp.mask_tiles_y = tiles_y;
+    mp.mask_blocks = (tiles_x * tiles_y + kMaskThreads - 1) / kMaskThreads;
+    for (int j = 0; j < nb; ++j) mp.order[j] = order[j];
+    march_global_kernel<<<mp.mask_blocks + items, kMaskThreads, 0, s>>>(mp);
+    if (cudaGetLastError() != cudaSuccess) return VR_ERR_CUDA;
     // direct front-to-back composite with the existing kernel
     static thread_local CompositeParams cp;
     std::memset(&cp, 0, sizeof(cp));
@@ -311,7 +301,6 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
     cp.tile_mask = masks;
     cp.tiles_x = tiles_x;
     cp.tiles_y = tiles_y;
-    if (launch_tile_masks(cp, s) != cudaSuccess) return VR_ERR_CUDA;
     if (launch_composite(cp, s) != cudaSuccess) return VR_ERR_CUDA;
     return VR_OK;
 }

@@ -11,14 +11,6 @@ namespace {
 
 using dev::over;
 
-// Stand-alone mask pass, for frames whose march does not write the masks.
-__global__ void __launch_bounds__(kMaskThreads) tile_mask_kernel(const __grid_constant__ CompositeParams p)
-{
-    dev::write_tile_mask(blockIdx.x * kMaskThreads + threadIdx.x, p.tiles_x, p.tiles_y, p.nb, p.order,
-                    [&](int b) { return make_int4(p.rect[b][0], p.rect[b][1], p.rect[b][2], p.rect[b][3]); },
-                    p.tile_mask);
-}
-
 // ---------------------------------------------------------------------------
 // Composite: one 32x8-thread block per kCompW x kCompTileH (32 x 8) image tile,
 // or a persistent grid whose blocks take tiles in turn; one thread per pixel.
@@ -178,14 +170,6 @@ cudaError_t launch_composite_images(const ImagesParams &p, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const long long blocks = std::min<long long>((p.pixels + 255) / 256, static_cast<long long>(sms) * 8);
     composite_images_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(p);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_tile_masks(const CompositeParams &p, cudaStream_t s)
-{
-    const int tiles = p.tiles_x * p.tiles_y;
-    if (tiles <= 0) return cudaSuccess;
-    tile_mask_kernel<<<(tiles + kMaskThreads - 1) / kMaskThreads, kMaskThreads, 0, s>>>(p);
     return cudaGetLastError();
 }
 

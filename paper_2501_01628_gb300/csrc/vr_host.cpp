@@ -441,7 +441,6 @@ vr_status prepare_frame(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, MarchParams &
     fr.tiles_x = (c.width + kCompW - 1) / kCompW;
     fr.tiles_y = (c.height + kCompTileH - 1) / kCompTileH;
     fr.pool_px = px + static_cast<long long>(fr.tiles_x) * fr.tiles_y;
-    fr.masks_ready = false;
     for (int a = 0; a < 3; ++a) {
         mp.eye[a] = static_cast<float>(c.eye[a]);
         mp.r[a] = static_cast<float>(B.r[a]);
@@ -543,7 +542,6 @@ vr_status march(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, cudaStream_t s, bool 
         VR_LAUNCH(ctx, launch_march(mp, vol->kind(), s, after_composite));
     }
     timing_end(ctx, t, s);
-    fr.masks_ready = true;
     return VR_OK;
 }
 
@@ -583,10 +581,6 @@ vr_status composite(vr_ctx ctx, vr_frame_s &fr, float4 *out, cudaStream_t s, int
     cp.tile_mask = reinterpret_cast<uint4 *>(fr.d_part + fr.total_px);
     cp.tiles_x = fr.tiles_x;
     cp.tiles_y = fr.tiles_y;
-    if (!fr.masks_ready) {  // a march that does not write them (meshes)
-        VR_LAUNCH(ctx, launch_tile_masks(cp, s));
-        fr.masks_ready = true;
-    }
     const int t = timing_begin(ctx, 1, s);
     if (sync) {
         cp.pool_done = sync->done;

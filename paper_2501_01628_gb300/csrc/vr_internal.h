@@ -19,18 +19,13 @@ enum StorageKind { kStoreF32 = 0, kStoreBF16 = 1, kStoreF16 = 2, kStoreBF16Oct =
 inline int storage_kind(vr_dtype t, bool octets) { return static_cast<int>(t) + (octets && t != VR_F32 ? 2 : 0); }
 constexpr int kMaxFactors = 8;
 
-// Work item of the no-allocation march: 16 x 8 pixels per 128-thread block,
-// four 8 x 4 warp packets (the other marches take the packet width as a
-// parameter, MarchParams::pw).
-constexpr int kTileW = 16;
-constexpr int kTileH = 8;
 // Composite: 256-thread blocks of 32 x 8 threads, one thread per pixel of a
 // 32 x 8 image tile with one brick mask per tile (the composite adjoint takes the
 // same tiles).
 constexpr int kCompW = 32;
 constexpr int kCompH = 8;
 constexpr int kCompTileH = kCompH;  // forward composite tile: kCompW x kCompTileH pixels
-constexpr int kMaskThreads = 128;                // threads (tiles) per block of the tile-mask pass
+constexpr int kMaskThreads = 128;                // threads (tiles) per mask block of a march grid
 
 // Brick storage index of quad (i, j, k): quads are grouped in 2x2x2 blocks of
 // 128 bytes (one L1 line for float32), blocks x-fastest; nbx, nby = blocks per
@@ -182,7 +177,7 @@ struct ImagesParams {
 // Pack of all bricks of a volume in one launch: block j of brick b (counted
 // from that brick's block_begin) writes the brick's storage quads
 // [j*kPackChunk, (j+1)*kPackChunk), in storage order.
-constexpr int kPackChunk = 2048;
+constexpr int kPackChunk = 1024;
 struct PackBrick {
     void *dst;             // the brick's storage
     long long quads;       // quads in the brick's storage (whole 2x2x2 blocks)
@@ -222,8 +217,6 @@ cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cuda
 // turn; 0: one block per tile.
 cudaError_t launch_composite(const CompositeParams &p, cudaStream_t s, int max_blocks = 0);
 cudaError_t launch_composite_images(const ImagesParams &p, cudaStream_t s);
-// Tile masks of p (p.tile_mask) for frames whose march did not write them.
-cudaError_t launch_tile_masks(const CompositeParams &p, cudaStream_t s);
 // Persistent batched kernel: cooperative launch of `blocks` blocks of 128 threads.
 cudaError_t launch_batch(const BatchParams &p, int kind, int blocks, cudaStream_t s);
 int batch_max_blocks_per_sm(int kind);

@@ -23,9 +23,35 @@ using dev::find_brick;
 // brick's storage (2x2x2 blocks of quads, blocks x-fastest), so a warp's writes
 // are contiguous. Quads of the padding that rounds a brick's storage up to
 // whole blocks are not written.
+//
+// Bound by memory: the volume once and the quads once (384^3: 0.23 + 0.93 GB). A
+// thread writes the two quads (i, i + 1) that share a sector: six loads for eight
+// voxels, one store. Its place in the storage is divided out once and then
+// stepped, and kPackUnroll pairs' loads are in flight together. 384^3 in 12
+// bricks: 0.190 ms, 6.0 TB/s (88% of a device copy); with one quad per thread 0.204,
+// and with two 64-bit divisions per quad, most of its instructions, 0.263.
 // ---------------------------------------------------------------------------
+constexpr int kPackThreads = 256, kPackUnroll = 2;
+static_assert(kPackChunk % (2 * kPackThreads * kPackUnroll) == 0, "whole rounds per block");
+// two consecutive elements at an address aligned to both
+__device__ __forceinline__ void store_pair(float4 *p, const float4 &a, const float4 &b)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void store_pair(uint4 *p, const uint4 &a, const uint4 &b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void store_pair(uint2 *p, const uint2 &a, const uint2 &b)
+{
+    *reinterpret_cast<uint4 *>(p) = make_uint4(a.x, a.y, b.x, b.y);
+}
 template <typename T>
-__global__ void __launch_bounds__(256) pack_kernel(const __grid_constant__ PackParams p)
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ PackParams p)
 {
     int lo = 0, hi = p.nb - 1;  // the block's brick (the same for all its threads)
     const int blk = blockIdx.x;
@@ -38,36 +64,65 @@ __global__ void __launch_bounds__(256) pack_kernel(const __grid_constant__ PackP
     using Q = typename Quad<T>::type;
     Q *dst = static_cast<Q *>(B.dst);
     const int qx = B.s[0] - 1, qy = B.s[1] - 1, nbx = B.s[0] / 2, nby = B.s[1] / 2;
-    const long long q0 = static_cast<long long>(blk - B.block_begin) * kPackChunk;
-    const long long q1 = min(q0 + kPackChunk, B.quads);
-    for (long long q = q0 + threadIdx.x; q < q1; q += 256) {
-        // inverse of quad_index
-        const long long bl = q >> 3;
-        const int bx = static_cast<int>(bl % nbx);
-        const long long rest = bl / nbx;
-        const int by = static_cast<int>(rest % nby);
-        const int bz = static_cast<int>(rest / nby);
-        const int lx = 2 * bx + static_cast<int>(q & 1), ly = 2 * by + static_cast<int>((q >> 1) & 1);
-        const int lz = 2 * bz + static_cast<int>((q >> 2) & 1);
-        if (lx >= qx || ly >= qy || lz >= B.s[2]) continue;
-        const int gx0 = min(max(B.lo[0] + lx - 1, 0), p.N[0] - 1);
-        const int gx1 = min(max(B.lo[0] + lx, 0), p.N[0] - 1);
-        const int gy0 = min(max(B.lo[1] + ly - 1, 0), p.N[1] - 1);
-        const int gy1 = min(max(B.lo[1] + ly, 0), p.N[1] - 1);
-        const int gz = min(max(B.lo[2] + lz - 1, 0), p.N[2] - 1);
-        const float *plane = p.src + static_cast<long long>(gz) * p.N[1] * p.N[0];
-        const float *r0 = plane + static_cast<long long>(gy0) * p.N[0];
-        const float *r1 = plane + static_cast<long long>(gy1) * p.N[0];
-        if constexpr (Quad<T>::octet) {  // plane lz and plane lz + 1 in one element
-            const int gz1 = min(max(B.lo[2] + lz, 0), p.N[2] - 1);
-            const float *plane1 = p.src + static_cast<long long>(gz1) * p.N[1] * p.N[0];
-            const float *s0 = plane1 + static_cast<long long>(gy0) * p.N[0];
-            const float *s1 = plane1 + static_cast<long long>(gy1) * p.N[0];
-            dst[q] = Quad<T>::make8(__ldg(r0 + gx0), __ldg(r0 + gx1), __ldg(r1 + gx0), __ldg(r1 + gx1),
-                                    __ldg(s0 + gx0), __ldg(s0 + gx1), __ldg(s1 + gx0), __ldg(s1 + gx1));
-        } else {
-            dst[q] = Quad<T>::make(__ldg(r0 + gx0), __ldg(r0 + gx1), __ldg(r1 + gx0), __ldg(r1 + gx1));
+    // a brick holds less than 2^31 quads; inverse of quad_index for the pair's first
+    unsigned q = static_cast<unsigned>(blk - B.block_begin) * kPackChunk + 2 * threadIdx.x;
+    const unsigned q1 = static_cast<unsigned>(B.quads);
+    const unsigned bl = q >> 3, rest = bl / static_cast<unsigned>(nbx);
+    int bx = static_cast<int>(bl - rest * nbx), bz = static_cast<int>(rest / static_cast<unsigned>(nby));
+    int by = static_cast<int>(rest) - bz * nby;
+    const int oy = static_cast<int>((q >> 1) & 1), oz = static_cast<int>((q >> 2) & 1);
+    constexpr int kPlanes = Quad<T>::octet ? 2 : 1;
+    for (int r = 0; r < kPackChunk / (2 * kPackThreads * kPackUnroll); ++r) {
+        float v[kPackUnroll][kPlanes][2][3];  // plane, row, x .. x + 2
+        bool in[kPackUnroll], both[kPackUnroll];
+#pragma unroll
+        for (int u = 0; u < kPackUnroll; ++u) {
+            const int lx = 2 * bx, ly = 2 * by + oy, lz = 2 * bz + oz;
+            in[u] = q + 2 * u * kPackThreads < q1 && lx < qx && ly < qy && lz < B.s[2];
+            both[u] = in[u] && lx + 1 < qx;
+            if (in[u]) {
+                int gx[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) gx[i] = min(max(B.lo[0] + lx - 1 + i, 0), p.N[0] - 1);
+#pragma unroll
+                for (int k = 0; k < kPlanes; ++k) {  // plane lz, and for octets plane lz + 1
+                    const int gz = min(max(B.lo[2] + lz - 1 + k, 0), p.N[2] - 1);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int gy = min(max(B.lo[1] + ly - 1 + j, 0), p.N[1] - 1);
+                        const float *row = p.src + (static_cast<long long>(gz) * p.N[1] + gy) * p.N[0];
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) v[u][k][j][i] = __ldg(row + gx[i]);
+                    }
+                }
+            }
+            bx += kPackThreads / 4;  // the next round's 2x2x2 block
+            while (bx >= nbx) {
+                bx -= nbx;
+                if (++by == nby) {
+                    by = 0;
+                    ++bz;
+                }
+            }
         }
+#pragma unroll
+        for (int u = 0; u < kPackUnroll; ++u) {
+            if (!in[u]) continue;
+            Q e[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float (&a)[2][3] = v[u][0], (&b)[2][3] = v[u][kPlanes - 1];
+                if constexpr (Quad<T>::octet)
+                    e[i] = Quad<T>::make8(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1], b[0][i], b[0][i + 1], b[1][i],
+                                          b[1][i + 1]);
+                else
+                    e[i] = Quad<T>::make(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1]);
+            }
+            Q *d = dst + q + 2 * u * kPackThreads;
+            if (both[u]) store_pair(d, e[0], e[1]);
+            else *d = e[0];
+        }
+        q += 2 * kPackThreads * kPackUnroll;
     }
 }
 
@@ -136,11 +191,11 @@ cudaError_t launch_pack(const PackParams &p, int kind, cudaStream_t s)
 {
     if (p.n_blocks <= 0) return cudaSuccess;
     switch (kind) {
-    case kStoreF32: pack_kernel<float><<<p.n_blocks, 256, 0, s>>>(p); break;
-    case kStoreBF16: pack_kernel<__nv_bfloat16><<<p.n_blocks, 256, 0, s>>>(p); break;
-    case kStoreF16: pack_kernel<__half><<<p.n_blocks, 256, 0, s>>>(p); break;
-    case kStoreBF16Oct: pack_kernel<dev::Octet<__nv_bfloat16>><<<p.n_blocks, 256, 0, s>>>(p); break;
-    case kStoreF16Oct: pack_kernel<dev::Octet<__half>><<<p.n_blocks, 256, 0, s>>>(p); break;
+    case kStoreF32: pack_kernel<float><<<p.n_blocks, kPackThreads, 0, s>>>(p); break;
+    case kStoreBF16: pack_kernel<__nv_bfloat16><<<p.n_blocks, kPackThreads, 0, s>>>(p); break;
+    case kStoreF16: pack_kernel<__half><<<p.n_blocks, kPackThreads, 0, s>>>(p); break;
+    case kStoreBF16Oct: pack_kernel<dev::Octet<__nv_bfloat16>><<<p.n_blocks, kPackThreads, 0, s>>>(p); break;
+    case kStoreF16Oct: pack_kernel<dev::Octet<__half>><<<p.n_blocks, kPackThreads, 0, s>>>(p); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

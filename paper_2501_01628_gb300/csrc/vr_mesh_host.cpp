@@ -515,7 +515,6 @@ vr_status vr_render_mesh_frame(vr_ctx ctx, vr_mesh mesh, float *out_rgba, int ou
     }();
     if (st != VR_OK) return give_back(st);
     timing_end(ctx, t, s);
-    fr.masks_ready = true;
     if (!pipe) return composite_to(ctx, fr, out_rgba, out_on_device, s);
     st = vr::host::composite_pipelined(ctx, fr, out_rgba, out_on_device, s, sync);
     if (st != VR_OK) return st;

@@ -757,7 +757,7 @@ def run_grad(a):
                                      "and all 256^3 voxels; value = forward samples per second of training steps"),
                 forward_ms_per_16_views=fwd_ms, backward_ms=ms - fwd_ms,
                 forward_samples_per_step=fwd_samples, loss=float(loss.detach()),
-                gpu_launches=a.steps * 16 * 7)
+                gpu_launches=a.steps * 16 * 9)
     print(json.dumps(line))
 
 

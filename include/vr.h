@@ -172,6 +172,12 @@ vr_status vr_volume_read_brick(vr_volume vol, int brick, void *dst, size_t bytes
  * device memory; it is copied, synchronously. */
 vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float vmin, float vmax,
                                    int on_device);
+/* The same for a table in device memory (16-byte aligned), in stream order: the
+ * library's table is written by a kernel on `stream`, without waiting on the
+ * host, for the renders launched on that stream afterwards. rgba_dev is read
+ * until that kernel is done. */
+vr_status vr_set_transfer_function_async(vr_ctx ctx, const float *rgba_dev, int n, float vmin, float vmax,
+                                         void *stream);
 vr_status vr_set_camera(vr_ctx ctx, const vr_camera *cam);
 /* step_voxels > 0 (default 0.5); ert_alpha in (0,1) enables early ray
  * termination per brick, >= 1 disables it (default 1). */

@@ -47,7 +47,12 @@ class Renderer:
         elif key != self._key:
             vr.vr_volume_update(self.vol, d)
         self._key = key
-        vr.vr_set_transfer_function(self.ctx, tf.detach().contiguous(), self.vmin, self.vmax)
+        table = tf.detach().contiguous()
+        if table.is_cuda and table.dtype == torch.float32 and table.data_ptr() % 16 == 0:
+            vr.vr_set_transfer_function_async(self.ctx, table, self.vmin, self.vmax)
+            table.record_stream(torch.cuda.current_stream())
+        else:
+            vr.vr_set_transfer_function(self.ctx, table, self.vmin, self.vmax)
         vr.vr_set_camera(self.ctx, cam)
 
     def render(self, tf: torch.Tensor, density: torch.Tensor, cam: dict) -> torch.Tensor:

@@ -497,7 +497,23 @@ __global__ void __launch_bounds__(256) grad_table_kernel(const float *copies, in
     }
 }
 
+__global__ void __launch_bounds__(128) table_pairs_kernel(const float4 *rgba, int n, float4 *pairs)
+{
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const float4 a = rgba[i], b = rgba[min(i + 1, n - 1)];
+    pairs[2 * i] = a;
+    pairs[2 * i + 1] = i + 1 < n ? make_float4(b.x - a.x, b.y - a.y, b.z - a.z, b.w - a.w)
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 }  // namespace
+
+cudaError_t launch_table_pairs(const float4 *rgba, int n, float4 *pairs, cudaStream_t s)
+{
+    table_pairs_kernel<<<(n + 127) / 128, 128, 0, s>>>(rgba, n, pairs);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_grad_groups(const GradParams &p, int kind, int groups, cudaStream_t s)
 {

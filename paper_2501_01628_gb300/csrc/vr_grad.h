@@ -74,4 +74,9 @@ cudaError_t launch_grad_samples(const GradParams &p, int groups, cudaStream_t s)
 cudaError_t launch_grad_voxels(const GradVoxelParams &p, cudaStream_t s);
 cudaError_t launch_grad_table(const float *tf_copies, int ntf, float *grad_tf, cudaStream_t s);
 
+// The table as the kernels read it, (T[i], T[i+1] - T[i]) pairs with the last
+// difference 0, from a device table (vr_set_transfer_function_async: fitting a
+// table changes it every step, and a copy to the host and back waits for the GPU).
+cudaError_t launch_table_pairs(const float4 *rgba, int n, float4 *pairs, cudaStream_t s);
+
 }  // namespace vr

@@ -1356,12 +1356,12 @@ vr_status vr_volume_read_brick(vr_volume vol, int brick, void *dst, size_t bytes
     return VR_OK;
 }
 
-vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float vmin, float vmax, int on_device)
+namespace {
+// Room for an n-entry device table and a valid scalar range.
+vr_status table_room(vr_ctx ctx, const float *rgba, int n, float vmin, float vmax)
 {
-    if (!ctx) return VR_ERR_ARG;
     if (!rgba || n < 2 || n > 1024 || !(vmax > vmin) || !std::isfinite(vmin) || !std::isfinite(vmax))
         return fail(ctx, VR_ERR_ARG, "bad transfer function");
-    DeviceGuard g(ctx->device);
     if (n > ctx->tf_cap) {
         cudaFree(ctx->d_tf);
         ctx->d_tf = nullptr;
@@ -1370,6 +1370,24 @@ vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float v
         VR_CUDA(ctx, vr::host::dev_malloc(&ctx->d_tf, 2 * static_cast<size_t>(n) * sizeof(float4)));
         ctx->tf_cap = n;
     }
+    return VR_OK;
+}
+
+void table_set(vr_ctx ctx, int n, float vmin, float vmax)
+{
+    ctx->ntf = n;
+    ctx->vmin = vmin;
+    ctx->vmax = vmax;
+    ctx->has_tf = true;
+}
+}  // namespace
+
+vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float vmin, float vmax, int on_device)
+{
+    if (!ctx) return VR_ERR_ARG;
+    DeviceGuard g(ctx->device);
+    vr_status st = table_room(ctx, rgba, n, vmin, vmax);
+    if (st != VR_OK) return st;
     // device table: (T[i], T[i+1] - T[i]) pairs in float32, last difference 0
     std::vector<float> t(4 * static_cast<size_t>(n)), pairs(8 * static_cast<size_t>(n));
     if (on_device)
@@ -1385,10 +1403,23 @@ vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float v
         }
     ctx->input_seq++;  // a pipelined march must not read the table across this upload
     VR_CUDA(ctx, cudaMemcpy(ctx->d_tf, pairs.data(), pairs.size() * sizeof(float), cudaMemcpyHostToDevice));
-    ctx->ntf = n;
-    ctx->vmin = vmin;
-    ctx->vmax = vmax;
-    ctx->has_tf = true;
+    table_set(ctx, n, vmin, vmax);
+    return VR_OK;
+}
+
+vr_status vr_set_transfer_function_async(vr_ctx ctx, const float *rgba_dev, int n, float vmin, float vmax,
+                                         void *stream)
+{
+    vr::host::TraceRange trace_("vr_set_transfer_function_async");
+    if (!ctx) return VR_ERR_ARG;
+    if (reinterpret_cast<uintptr_t>(rgba_dev) & 15) return fail(ctx, VR_ERR_ARG, "table must be 16-byte aligned");
+    DeviceGuard g(ctx->device);
+    vr_status st = table_room(ctx, rgba_dev, n, vmin, vmax);
+    if (st != VR_OK) return st;
+    ctx->input_seq++;  // a pipelined march must not read the table across this kernel
+    VR_LAUNCH(ctx, launch_table_pairs(reinterpret_cast<const float4 *>(rgba_dev), n, ctx->d_tf,
+                                      static_cast<cudaStream_t>(stream)));
+    table_set(ctx, n, vmin, vmax);
     return VR_OK;
 }
 

@@ -41,7 +41,7 @@ EXPORTS = (
     "vr_set_host_output_async", "vr_mesh_create", "vr_mesh_release", "vr_mesh_info",
     "vr_render_mesh_frame", "vr_debug_inject_fault", "vr_batch_debug_wait", "vr_set_march_staging",
     "vr_volume_create_share", "vr_composite_images", "vr_set_cell_layout", "vr_set_frame_pipelining",
-    "vr_debug_pipeline_gap",
+    "vr_debug_pipeline_gap", "vr_set_transfer_function_async",
 )
 
 
@@ -79,6 +79,7 @@ _SIG = {
     "vr_volume_info": (_I, [_P, _P, _P, _P]),
     "vr_volume_read_brick": (_I, [_P, _I, _P, ctypes.c_size_t]),
     "vr_set_transfer_function": (_I, [_P, _P, _I, ctypes.c_float, ctypes.c_float, _I]),
+    "vr_set_transfer_function_async": (_I, [_P, _P, _I, ctypes.c_float, ctypes.c_float, _P]),
     "vr_set_camera": (_I, [_P, ctypes.POINTER(vr_camera)]),
     "vr_set_render_params": (_I, [_P, ctypes.c_float, ctypes.c_float]),
     "vr_set_composite_schedule": (_I, [_P, _I, _P]),
@@ -446,6 +447,18 @@ def vr_set_transfer_function(ctx, rgba, vmin: float, vmax: float):
     n = int(keep.shape[0])
     _check(lib().vr_set_transfer_function(ctx, ptr, n, float(vmin), float(vmax), on_dev), ctx,
            "vr_set_transfer_function")
+    _tf_len[_key(ctx)] = n
+
+
+def vr_set_transfer_function_async(ctx, rgba, vmin: float, vmax: float, stream=None):
+    """vr_set_transfer_function of a CUDA float32 (n, 4) tensor in stream order,
+    without waiting on the host."""
+    ptr, _, keep = _array(rgba, "transfer function", ndim=2, device=True)
+    if keep.shape[1] != 4:
+        raise ValueError("transfer function must be (n, 4) RGBA")
+    n = int(keep.shape[0])
+    _check(lib().vr_set_transfer_function_async(ctx, ptr, n, float(vmin), float(vmax), _stream(stream)), ctx,
+           "vr_set_transfer_function_async")
     _tf_len[_key(ctx)] = n
 
 

@@ -309,6 +309,9 @@ vr_status vr_frame_partial(vr_frame fr, int brick, const float **dev_ptr);
  * schedule into out_rgba (device memory if out_on_device, else host memory; a
  * host output makes the call synchronous). */
 vr_status vr_composite(vr_ctx ctx, vr_frame fr, float *out_rgba, int out_on_device, void *stream);
+/* Waits for the device. The context keeps the last released frame's memory (up
+ * to 1 GiB) for the next vr_render_partials; vr_destroy, or an allocation of the
+ * context that finds no room, gives it back. */
 vr_status vr_frame_release(vr_frame fr);
 /* Sec. 3: the ranks' images end up composited into one framebuffer. out_dev =
  * images_dev[0] over images_dev[1] over ... over images_dev[n-1], pixel by pixel

@@ -37,6 +37,19 @@ bool fault_now(int kind)
     return true;
 }
 
+cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes)
+{
+    cudaError_t e = dev_malloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->spare) {
+        cudaGetLastError();
+        cudaFree(ctx->spare);
+        ctx->spare = nullptr;
+        ctx->spare_px = 0;
+        e = dev_malloc(p, bytes);
+    }
+    return e;
+}
+
 size_t elem_size(vr_dtype t) { return t == VR_F32 ? 4 : 2; }
 // bytes of one xy-quad (four voxels) in device storage
 // bytes of one storage element: an xy-quad (four voxels), or an octet (both
@@ -378,11 +391,16 @@ cudaError_t pack_bricks(vr_volume vol, const float *dsrc, cudaStream_t s)
 vr_status ensure_frame(vr_ctx ctx, vr_frame_s &fr, long long px)
 {
     if (px <= fr.cap_px) return VR_OK;
+    if (!fr.owned_by_ctx && !fr.d_part && px <= ctx->spare_px) {
+        std::swap(fr.d_part, ctx->spare);
+        std::swap(fr.cap_px, ctx->spare_px);
+        return VR_OK;
+    }
     const long long want = std::max(px, fr.cap_px + fr.cap_px / 4);
     if (fr.d_part) cudaFree(fr.d_part);
     fr.d_part = nullptr;
     fr.cap_px = 0;
-    VR_CUDA(ctx, vr::host::dev_malloc(&fr.d_part, static_cast<size_t>(want) * sizeof(float4)));
+    VR_CUDA(ctx, vr::host::dev_malloc(ctx, &fr.d_part, static_cast<size_t>(want) * sizeof(float4)));
     fr.cap_px = want;
     return VR_OK;
 }
@@ -603,7 +621,7 @@ vr_status host_staging(vr_ctx ctx, long long px, cudaStream_t s, float4 **buf, i
             if (ctx->d_img) cudaFree(ctx->d_img);
             ctx->d_img = nullptr;
             ctx->img_cap = 0;
-            VR_CUDA(ctx, vr::host::dev_malloc(&ctx->d_img, static_cast<size_t>(px) * sizeof(float4)));
+            VR_CUDA(ctx, vr::host::dev_malloc(ctx, &ctx->d_img, static_cast<size_t>(px) * sizeof(float4)));
             ctx->img_cap = px;
         }
         *buf = ctx->d_img;
@@ -625,7 +643,7 @@ vr_status host_staging(vr_ctx ctx, long long px, cudaStream_t s, float4 **buf, i
         }
         ctx->img2_cap = 0;
         for (int i = 0; i < 2; ++i)
-            VR_CUDA(ctx, vr::host::dev_malloc(&ctx->d_img2[i], static_cast<size_t>(px) * sizeof(float4)));
+            VR_CUDA(ctx, vr::host::dev_malloc(ctx, &ctx->d_img2[i], static_cast<size_t>(px) * sizeof(float4)));
         ctx->img2_cap = px;
     }
     const int k = ctx->img_next;
@@ -907,6 +925,7 @@ vr_status vr_destroy(vr_ctx ctx)
     cudaFree(ctx->d_counter);
     cudaFree(ctx->d_error);
     cudaFree(ctx->d_grad);
+    cudaFree(ctx->spare);
     cudaFree(ctx->frame.d_part);
     cudaFree(ctx->frame2.d_part);
     cudaFree(ctx->d_pool_done);
@@ -1038,7 +1057,7 @@ vr_status create_volume(vr_ctx ctx, const int dims[3], vr_dtype storage, const v
     off_bytes = std::max(off_bytes, 256LL);
     DeviceGuard g(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    VR_CUDA(ctx, vr::host::dev_malloc(&vol->d_data, static_cast<size_t>(off_bytes)));
+    VR_CUDA(ctx, vr::host::dev_malloc(ctx, &vol->d_data, static_cast<size_t>(off_bytes)));
     vol->bytes = vol->quad_bytes = off_bytes;
     if (ctx->staging && storage == VR_F32) {
         // scalar copy for the staged march: rows padded to 4 elements (16 bytes),
@@ -1055,7 +1074,7 @@ vr_status create_volume(vr_ctx ctx, const int dims[3], vr_dtype storage, const v
             off = (off + 31) & ~31LL;
         }
         off = std::max(off, 32LL);
-        const cudaError_t es2 = vr::host::dev_malloc(&vol->d_scalar, static_cast<size_t>(off) * sizeof(float));
+        const cudaError_t es2 = vr::host::dev_malloc(ctx, &vol->d_scalar, static_cast<size_t>(off) * sizeof(float));
         if (es2 != cudaSuccess) {
             cudaFree(vol->d_data);
             return cuda_fail(ctx, es2, "scalar brick copy");
@@ -1066,7 +1085,7 @@ vr_status create_volume(vr_ctx ctx, const int dims[3], vr_dtype storage, const v
     float *tmp = nullptr;
     const size_t nvox = static_cast<size_t>(dims[0]) * dims[1] * dims[2];
     if (!src_on_device) {
-        cudaError_t e = vr::host::dev_malloc(&tmp, nvox * sizeof(float));
+        cudaError_t e = vr::host::dev_malloc(ctx, &tmp, nvox * sizeof(float));
         if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, src, nvox * sizeof(float), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) {
             cudaFree(tmp);
@@ -1117,7 +1136,7 @@ vr_status vr_volume_update(vr_volume vol, const float *src, int src_on_device, v
     const float *dsrc = src;
     float *tmp = nullptr;
     if (!src_on_device) {
-        VR_CUDA(ctx, vr::host::dev_malloc(&tmp, nvox * sizeof(float)));
+        VR_CUDA(ctx, vr::host::dev_malloc(ctx, &tmp, nvox * sizeof(float)));
         cudaError_t e = cudaMemcpyAsync(tmp, src, nvox * sizeof(float), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) {
             cudaFree(tmp);
@@ -1142,7 +1161,7 @@ vr_status vr_volume_update_async(vr_volume vol, const float *src, int src_on_dev
     const size_t nvox = static_cast<size_t>(vol->dims[0]) * vol->dims[1] * vol->dims[2];
     const float *dsrc = src;
     if (!src_on_device) {
-        if (!vol->d_staging) VR_CUDA(ctx, vr::host::dev_malloc(&vol->d_staging, nvox * sizeof(float)));
+        if (!vol->d_staging) VR_CUDA(ctx, vr::host::dev_malloc(ctx, &vol->d_staging, nvox * sizeof(float)));
         VR_CUDA(ctx, cudaMemcpyAsync(vol->d_staging, src, nvox * sizeof(float), cudaMemcpyHostToDevice, s));
         dsrc = vol->d_staging;
     }
@@ -1237,7 +1256,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         cudaFree(ctx->d_grad);
         ctx->d_grad = nullptr;
         ctx->grad_cap = 0;
-        const cudaError_t e = vr::host::dev_malloc(&ctx->d_grad, need);
+        const cudaError_t e = vr::host::dev_malloc(ctx, &ctx->d_grad, need);
         if (e == cudaSuccess) {
             ctx->grad_cap = need;
             break;
@@ -1256,7 +1275,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     gp.grad_quads = nullptr;
     const long long quads = vol->quad_bytes / static_cast<long long>(quad_size(vol->dtype, vol->octets));
     if (grad_density_dev && view_segs * kGradSeg > kGradQuadsRatio * quads) {
-        if (!vol->d_gquads && vr::host::dev_malloc(&vol->d_gquads, quads * sizeof(float4)) != cudaSuccess)
+        if (!vol->d_gquads && vr::host::dev_malloc(ctx, &vol->d_gquads, quads * sizeof(float4)) != cudaSuccess)
             cudaGetLastError();  // no room: reductions straight into the voxels
         gp.grad_quads = vol->d_gquads;
     }
@@ -1367,7 +1386,7 @@ vr_status table_room(vr_ctx ctx, const float *rgba, int n, float vmin, float vma
         ctx->d_tf = nullptr;
         ctx->tf_cap = 0;
         ctx->has_tf = false;
-        VR_CUDA(ctx, vr::host::dev_malloc(&ctx->d_tf, 2 * static_cast<size_t>(n) * sizeof(float4)));
+        VR_CUDA(ctx, vr::host::dev_malloc(ctx, &ctx->d_tf, 2 * static_cast<size_t>(n) * sizeof(float4)));
         ctx->tf_cap = n;
     }
     return VR_OK;
@@ -1518,9 +1537,17 @@ vr_status vr_composite(vr_ctx ctx, vr_frame fr, float *out_rgba, int out_on_devi
 vr_status vr_frame_release(vr_frame fr)
 {
     if (!fr || fr->owned_by_ctx) return VR_ERR_ARG;
-    DeviceGuard g(fr->ctx->device);
+    vr_ctx ctx = fr->ctx;
+    DeviceGuard g(ctx->device);
+    if (fr->cap_px > ctx->spare_px && fr->cap_px * static_cast<long long>(sizeof(float4)) <= kSpareBytes) {
+        // nothing may still use the memory when the next frame takes it: kernels of
+        // any stream, the caller's own on vr_frame_partial's pointers among them
+        cudaDeviceSynchronize();
+        std::swap(fr->d_part, ctx->spare);
+        std::swap(fr->cap_px, ctx->spare_px);
+    }
     cudaFree(fr->d_part);
-    fr->ctx->live_objects--;
+    ctx->live_objects--;
     delete fr;
     return VR_OK;
 }

@@ -411,10 +411,10 @@ vr_status vr_mesh_create(vr_ctx ctx, const int dims[3], const vr_partition *part
         cudaFree(m->d_nodes);
         cudaFree(m->d_start);
     };
-    cudaError_t e = vr::host::dev_malloc(&m->d_rec, rec_bytes);
-    if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_nbr, nbr_bytes);
-    if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_nodes, node_bytes);
-    if (e == cudaSuccess) e = vr::host::dev_malloc(&m->d_start, start_bytes);
+    cudaError_t e = vr::host::dev_malloc(ctx, &m->d_rec, rec_bytes);
+    if (e == cudaSuccess) e = vr::host::dev_malloc(ctx, &m->d_nbr, nbr_bytes);
+    if (e == cudaSuccess) e = vr::host::dev_malloc(ctx, &m->d_nodes, node_bytes);
+    if (e == cudaSuccess) e = vr::host::dev_malloc(ctx, &m->d_start, start_bytes);
     for (int b = 0; e == cudaSuccess && b < nb; ++b) {
         const BrickBuild &B = bricks[b];
         e = cudaMemcpy(m->d_rec + kMeshRec * m->rec_base[b], B.rec.data(), B.rec.size() * sizeof(float4),

@@ -56,17 +56,22 @@ struct GradBrick {
 struct GradCell {
     unsigned bx, by, bz;
     float wx, wy, wz;
-    // quad indices of the cell's planes k and k + 1
-    __device__ __forceinline__ void quads(const GradBrick &G, unsigned &c, unsigned &c1) const
+    // quad index of the cell's plane k, and of plane k + 1
+    __device__ __forceinline__ unsigned place(const GradBrick &G) const
     {
-        c = bz * G.az + G.c0;
+        unsigned c = bz * G.az + G.c0;
         c = by * G.ay + c;
         c = bx * 4u + c;
         c = (bx & 1u) * (0u - 3u) + c;
         c = (by & 1u) * G.py + c;
-        c = (bz & 1u) * G.pz + c;
-        c1 = min(c + 4u + (bz & 1u) * G.dz, G.last);
-        c = min(c, G.last);
+        return (bz & 1u) * G.pz + c;
+    }
+    __device__ __forceinline__ unsigned quad(const GradBrick &G) const { return min(place(G), G.last); }
+    __device__ __forceinline__ void quads(const GradBrick &G, unsigned &c, unsigned &c1) const
+    {
+        const unsigned at = place(G);
+        c = min(at, G.last);
+        c1 = min(at + 4u + (bz & 1u) * G.dz, G.last);
     }
 };
 
@@ -78,9 +83,8 @@ __device__ __forceinline__ unsigned grad_floor(float v, float &w)
     return __float_as_uint(y);
 }
 
-__device__ __forceinline__ void grad_cell(const dev::OwnedRun &run, int kk, GradCell &q)
+__device__ __forceinline__ void grad_cell(const dev::OwnedRun &run, float h, GradCell &q)
 {
-    const float h = static_cast<float>(kk) + 0.5f;
     q.bx = grad_floor(fmaf(h, run.step[0], run.base[0]), q.wx);
     q.by = grad_floor(fmaf(h, run.step[1], run.base[1]), q.wy);
     q.bz = grad_floor(fmaf(h, run.step[2], run.base[2]), q.wz);
@@ -92,7 +96,7 @@ __device__ __forceinline__ float grad_value(const MarchParams &m, const typename
                                             const GradBrick &G, const dev::OwnedRun &run, int kk)
 {
     GradCell q;
-    grad_cell(run, kk, q);
+    grad_cell(run, static_cast<float>(kk) + 0.5f, q);
     unsigned c, c1;
     q.quads(G, c, c1);
     float4 a0, a1;
@@ -282,9 +286,10 @@ __global__ void __launch_bounds__(256) grad_scan_kernel(const __grid_constant__ 
     }
 }
 
-__device__ __forceinline__ void red_v4(float *dst, float a, float b, float c, float d)
+__device__ __forceinline__ void red_v4(float4 *dst, const float (&v)[4])
 {
-    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(a), "f"(b), "f"(c), "f"(d)
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(v[0]), "f"(v[1]),
+                 "f"(v[2]), "f"(v[3])
                  : "memory");
 }
 
@@ -292,16 +297,18 @@ __device__ __forceinline__ void red_v4(float *dst, float a, float b, float c, fl
 // last sample is repeated with T and opacity 0, so nothing branches on the
 // length and the segment's loads are in flight together. Gradients of
 // consecutive samples in one cell, and in one table interval, are summed in
-// registers before they are added to memory: the table with two 16-byte
-// reductions per interval into the block's copy (float atomics in shared memory
-// are compare-and-swap loops), the voxels with two 16-byte reductions per cell
-// into quads laid out as the brick's own (QUADS; grad_voxels_kernel then adds
-// them to the voxels), or with one reduction per corner on the original
-// volume's indexing (halo copies alias their neighbours' voxels).
-// Bound by issue (43%) and by the reductions on their way to L2 (37% of its
-// rate): 0.46 ms for a 512^2 view of a 256^3 volume, where one thread per run with
-// shared-memory table gradients and three samplings took 2.1 ms. 4, 6 and 7
-// blocks per SM measured the same within 2%.
+// registers before they are added to memory: the table with a 16-byte
+// reduction per entry left behind into one of the copies (float atomics in shared
+// memory are compare-and-swap loops), the voxels with a 16-byte reduction per
+// quad left behind into quads laid out as the brick's own (QUADS;
+// grad_voxels_kernel then adds them to the voxels), or with one reduction per
+// corner on the original volume's indexing (halo copies alias their neighbours'
+// voxels).
+// Bound by issue (63% of slots) at 23 of 32 lanes, then by the reductions on their
+// way to L2 (35% of its rate): 0.37 ms for a 512^2 view of a 256^3 volume (0.46 with
+// both entries and both planes added at every change; one thread per run with
+// shared-memory table gradients and three samplings took 2.1 ms). 4 and 6 blocks
+// per SM measured the same and 4% more.
 template <bool QUADS>
 __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_constant__ GradParams p)
 {
@@ -317,56 +324,73 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
     const float xmax = static_cast<float>(m.ntf - 1);
     // neighbouring lanes, whose samples often share an interval, add into different copies
     const unsigned which = ((blockIdx.x + blockIdx.y) * kGradLaneCopies + threadIdx.x % kGradLaneCopies) % kGradCopies;
-    float *copy = p.tf_copies + static_cast<long long>(which) * m.ntf * kGradEntry;
+    float4 *copy = reinterpret_cast<float4 *>(p.tf_copies) + static_cast<long long>(which) * (m.ntf + 1);
     const bool voxels = QUADS || p.grad_vol;
-    unsigned cur_x = 0, cur_y = 0, cur_z = 0;  // no cell: floors' bits are never 0
-    float acc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-    int cur_ti = -1;
+    float4 *gquads = QUADS ? p.grad_quads + B.base : nullptr;
+    // the cell being summed: quad index of its lower plane, floors (0: no cell)
+    unsigned cur_c = 0, cur_x = 0, cur_y = 0, cur_z = 0;
+    float lower[4], upper[4];
+    int cur_ti = -4;  // the table interval being summed (negative: none)
     float at0[4], at1[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) at0[c] = at1[c] = 0.0f;
-    auto flush_tf = [&]() {
-        if (cur_ti < 0) return;
-        float *d = copy + cur_ti * kGradEntry;
-        red_v4(d, at0[0], at0[1], at0[2], at0[3]);
-        red_v4(d + 4, at1[0], at1[1], at1[2], at1[3]);
-    };
-    auto flush = [&]() {
-        if (cur_x == 0) return;
-        if constexpr (QUADS) {
-            GradCell q;
-            q.bx = cur_x;
-            q.by = cur_y;
-            q.bz = cur_z;
-            unsigned c, c1;
-            q.quads(G, c, c1);
-            float4 *dst = p.grad_quads + B.base;
-            red_v4(reinterpret_cast<float *>(dst + c), acc[0], acc[1], acc[2], acc[3]);
-            red_v4(reinterpret_cast<float *>(dst + c1), acc[4], acc[5], acc[6], acc[7]);
-        } else {
-            const int i = static_cast<int>(cur_x - dev::kFloorBits), j = static_cast<int>(cur_y - dev::kFloorBits),
-                      k = static_cast<int>(cur_z - dev::kFloorBits);
-            const int gx0 = min(max(B.lo[0] - 1 + i, 0), p.N[0] - 1), gx1 = min(max(B.lo[0] + i, 0), p.N[0] - 1);
-            const int gy0 = min(max(B.lo[1] - 1 + j, 0), p.N[1] - 1), gy1 = min(max(B.lo[1] + j, 0), p.N[1] - 1);
-            const int gz0 = min(max(B.lo[2] - 1 + k, 0), p.N[2] - 1), gz1 = min(max(B.lo[2] + k, 0), p.N[2] - 1);
-            const long long nx = p.N[0], nxy = static_cast<long long>(p.N[0]) * p.N[1];
-            float *gv = p.grad_vol;
-            atomicAdd(gv + gz0 * nxy + gy0 * nx + gx0, acc[0]);
-            atomicAdd(gv + gz0 * nxy + gy0 * nx + gx1, acc[1]);
-            atomicAdd(gv + gz0 * nxy + gy1 * nx + gx0, acc[2]);
-            atomicAdd(gv + gz0 * nxy + gy1 * nx + gx1, acc[3]);
-            atomicAdd(gv + gz1 * nxy + gy0 * nx + gx0, acc[4]);
-            atomicAdd(gv + gz1 * nxy + gy0 * nx + gx1, acc[5]);
-            atomicAdd(gv + gz1 * nxy + gy1 * nx + gx0, acc[6]);
-            atomicAdd(gv + gz1 * nxy + gy1 * nx + gx1, acc[7]);
+    for (int c = 0; c < 4; ++c) lower[c] = upper[c] = at0[c] = at1[c] = 0.0f;
+    // on to interval ti: an entry that the next interval shares stays in registers
+    auto next_interval = [&](int ti) {
+        const bool up = ti - cur_ti == 1, down = cur_ti - ti == 1;
+        if (cur_ti >= 0) {
+            if (!down) red_v4(copy + cur_ti, at0);
+            if (!up) red_v4(copy + cur_ti + 1, at1);
         }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float lo = at0[c], hi = at1[c];
+            at0[c] = up ? hi : 0.0f;
+            at1[c] = down ? lo : 0.0f;
+        }
+        cur_ti = ti;
+    };
+    // on to cell q, likewise for the plane that a step along z shares
+    auto next_cell = [&](const GradCell &q) {
+        const bool column = q.bx == cur_x && q.by == cur_y;
+        const bool up = QUADS && column && q.bz - cur_z == 1u, down = QUADS && column && cur_z - q.bz == 1u;
+        if (cur_x != 0) {
+            if constexpr (QUADS) {
+                if (!down) red_v4(gquads + cur_c, lower);
+                if (!up) red_v4(gquads + min(cur_c + 4u + (cur_z & 1u) * G.dz, G.last), upper);
+            } else {
+                const int i = static_cast<int>(cur_x - dev::kFloorBits), j = static_cast<int>(cur_y - dev::kFloorBits),
+                          k = static_cast<int>(cur_z - dev::kFloorBits);
+                const int gx0 = min(max(B.lo[0] - 1 + i, 0), p.N[0] - 1), gx1 = min(max(B.lo[0] + i, 0), p.N[0] - 1);
+                const int gy0 = min(max(B.lo[1] - 1 + j, 0), p.N[1] - 1), gy1 = min(max(B.lo[1] + j, 0), p.N[1] - 1);
+                const int gz0 = min(max(B.lo[2] - 1 + k, 0), p.N[2] - 1), gz1 = min(max(B.lo[2] + k, 0), p.N[2] - 1);
+                const long long nx = p.N[0], nxy = static_cast<long long>(p.N[0]) * p.N[1];
+                float *gv = p.grad_vol;
+                atomicAdd(gv + gz0 * nxy + gy0 * nx + gx0, lower[0]);
+                atomicAdd(gv + gz0 * nxy + gy0 * nx + gx1, lower[1]);
+                atomicAdd(gv + gz0 * nxy + gy1 * nx + gx0, lower[2]);
+                atomicAdd(gv + gz0 * nxy + gy1 * nx + gx1, lower[3]);
+                atomicAdd(gv + gz1 * nxy + gy0 * nx + gx0, upper[0]);
+                atomicAdd(gv + gz1 * nxy + gy0 * nx + gx1, upper[1]);
+                atomicAdd(gv + gz1 * nxy + gy1 * nx + gx0, upper[2]);
+                atomicAdd(gv + gz1 * nxy + gy1 * nx + gx1, upper[3]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float lo = lower[c], hi = upper[c];
+            lower[c] = up ? hi : 0.0f;
+            upper[c] = down ? lo : 0.0f;
+        }
+        cur_x = q.bx;
+        cur_y = q.by;
+        cur_z = q.bz;
+        if constexpr (QUADS) cur_c = q.quad(G);
     };
     const float2 ends = p.group[p.goff[it.b] + blockIdx.y * it.area + it.pixel];
     float lamT = ends.x;
     for (int s = it.s1 - 1; s >= it.s0; --s) {
         const int k0 = it.run.ka + s * kGradSeg, left = it.run.kb - k0;  // samples 0 .. min(left, kGradSeg - 1)
+        const float h0 = static_cast<float>(k0) + 0.5f;
         const float *x = p.x + p.soff[it.b] * kGradSeg + s * it.area * kGradSeg + it.pixel;
         float T = ends.y * p.front[p.soff[it.b] + s * it.area + it.pixel];
         float xs[kGradSeg], Ts[kGradSeg];
@@ -393,12 +417,7 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
             const float g4[4] = {it.g.x * ta, it.g.y * ta, it.g.z * ta, Ts[j] * (gc - lamT)};
             lamT = lamT * (1.0f - a) + a * gc;
             // table: rgba = (1-w) T[i] + w T[i+1]
-            if (ti != cur_ti) {
-                flush_tf();
-                cur_ti = ti;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) at0[c] = at1[c] = 0.0f;
-            }
+            if (ti != cur_ti) next_interval(ti);
             const float w0 = 1.0f - w;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -406,33 +425,26 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
                 at1[c] = fmaf(w, g4[c], at1[c]);
             }
             // scalar: ds = (g . (T[i+1] - T[i])) dx/ds where the table coordinate is not clamped
-            if (voxels && xj > 0.0f && xj < xmax) {
+            if (voxels && j <= left && xj > 0.0f && xj < xmax) {
                 const float ds = (g4[0] * de.x + g4[1] * de.y + g4[2] * de.z + g4[3] * de.w) * m.tf_scale;
                 GradCell q;
-                grad_cell(it.run, k0 + min(j, left), q);
-                if (q.bx != cur_x || q.by != cur_y || q.bz != cur_z) {
-                    flush();
-                    cur_x = q.bx;
-                    cur_y = q.by;
-                    cur_z = q.bz;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-                }
+                grad_cell(it.run, h0 + static_cast<float>(j), q);
+                if (q.bx != cur_x || q.by != cur_y || q.bz != cur_z) next_cell(q);
                 const float ux = 1.0f - q.wx, uy = 1.0f - q.wy, uz = 1.0f - q.wz;
                 const float dz0 = ds * uz, dz1 = ds * q.wz;
-                acc[0] = fmaf(dz0, ux * uy, acc[0]);
-                acc[1] = fmaf(dz0, q.wx * uy, acc[1]);
-                acc[2] = fmaf(dz0, ux * q.wy, acc[2]);
-                acc[3] = fmaf(dz0, q.wx * q.wy, acc[3]);
-                acc[4] = fmaf(dz1, ux * uy, acc[4]);
-                acc[5] = fmaf(dz1, q.wx * uy, acc[5]);
-                acc[6] = fmaf(dz1, ux * q.wy, acc[6]);
-                acc[7] = fmaf(dz1, q.wx * q.wy, acc[7]);
+                lower[0] = fmaf(dz0, ux * uy, lower[0]);
+                lower[1] = fmaf(dz0, q.wx * uy, lower[1]);
+                lower[2] = fmaf(dz0, ux * q.wy, lower[2]);
+                lower[3] = fmaf(dz0, q.wx * q.wy, lower[3]);
+                upper[0] = fmaf(dz1, ux * uy, upper[0]);
+                upper[1] = fmaf(dz1, q.wx * uy, upper[1]);
+                upper[2] = fmaf(dz1, ux * q.wy, upper[2]);
+                upper[3] = fmaf(dz1, q.wx * q.wy, upper[3]);
             }
         }
     }
-    if (voxels) flush();
-    flush_tf();
+    if (voxels) next_cell(GradCell{});
+    next_interval(-4);
 }
 
 // Step 4 (QUADS): every haloed voxel of every brick sums its share of the four
@@ -477,14 +489,12 @@ __global__ void __launch_bounds__(256) grad_table_kernel(const float *copies, in
 {
     __shared__ float s_sum[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int v = blockIdx.x * 32 + lane, e = v >> 2, c = v & 3;
+    const int v = blockIdx.x * 32 + lane;
     float sum = 0.0f;
     if (v < 4 * ntf) {
 #pragma unroll
         for (int k = warp; k < kGradCopies; k += 8) {
-            const float *d = copies + (static_cast<long long>(k) * ntf + e) * kGradEntry;
-            sum += d[c];
-            if (e > 0) sum += d[4 + c - kGradEntry];
+            sum += copies[static_cast<long long>(k) * 4 * (ntf + 1) + v];
         }
     }
     s_sum[warp][lane] = sum;

@@ -13,21 +13,19 @@ namespace vr {
 constexpr int kGradSeg = 8;
 constexpr int kGradGroup = 8;
 constexpr int kGradMaxRun = 4096;
-// Copies of the table gradient, spread over blocks and lanes so that few
-// reductions meet on one entry. 256^3 volume, 4 views of 512^2, ms per training
-// step: 7.29 with 16 copies by block, 6.44 with 64, 6.21 with 256, 6.15 with
-// 1024 by block and lane % 8, 6.66 with 4096 by block and lane.
+// Copies of the table gradient ((ntf + 1) x 4 floats each), spread over blocks and
+// lanes so that few reductions meet on one entry. 256^3 volume, 4 views of 512^2, ms
+// per training step: 7.29 with 16 copies by block, 6.44 with 64, 6.21 with 256, 6.15
+// with 1024 by block and lane % 8, 6.66 with 4096 by block and lane.
 constexpr int kGradCopies = 512;
 constexpr int kGradLaneCopies = 8;
-constexpr int kGradEntry = 8;      // floats per table interval in a copy: d/dT[i], d/dT[i+1]
-// Voxel gradients go through quads (two 16-byte reductions per cell, then one pass
-// over the volume's quads) when the view's samples, bounded by rect areas times
-// longest runs, are over this many times the quads, else straight into the voxels
-// (eight reductions per cell). One view, 8 bricks, us per training step quads /
-// direct: 256^3 at 128^2 (ratio 0.8) 1240 / 1147, at 256^2 (3) 1413 / 1319, at
-// 384^2 (7) 1545 / 1550; 128^3 at 256^2 (12) 1045 / 1063; 64^3 at 256^2 (47) 953 /
-// 1001; 256^3, four views at 512^2 (12) 6450 / 7160.
-constexpr long long kGradQuadsRatio = 6;
+// Voxel gradients go through quads (at most two 16-byte reductions per cell, then
+// one pass over the volume's quads) when the view's samples, bounded by rect areas
+// times longest runs, are over this many times the quads, else straight into the
+// voxels (eight reductions per cell). One view, 8 bricks, us per training step quads
+// / direct: 256^3 at 256^2 (ratio 1.6) 1362 / 1287, at 384^2 (3.6 to 4.4) 1500 / 1541;
+// 128^3 at 256^2 (6.4) 1025 / 1099; 256^3, four views at 512^2 (5.8 to 7.4) 5320 / 6010.
+constexpr long long kGradQuadsRatio = 4;
 constexpr long long kGradBandBytes = 1LL << 30;  // per-sample workspace of one band of image rows
 
 struct GradParams {
@@ -41,7 +39,7 @@ struct GradParams {
     long long soff[kMaxBricks], goff[kMaxBricks];
     int nseg[kMaxBricks];         // segments kept per pixel
     unsigned short *count;        // per (brick, pixel), at BrickLaunch::poff: groups of the run
-    float *tf_copies;             // kGradCopies x ntf x kGradEntry, zeroed before the launches
+    float *tf_copies;             // kGradCopies x (ntf + 1) x 4, zeroed before the launches
     float *grad_vol;              // Nz x Ny x Nx, or null
     float4 *grad_quads;           // quads of voxel gradients laid out as the bricks', or null
                                   // (reductions straight into grad_vol)

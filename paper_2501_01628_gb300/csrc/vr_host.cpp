@@ -1189,7 +1189,6 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     // runs are refused (the last segment then takes the rest)
     const int nb = fr.nb;
     int groups = 0;
-    long long row_segs = 0;  // segments of one full image row
     int ngroup[kMaxBricks];
     for (int b = 0; b < nb; ++b) {
         const int *bx = &vol->boxes[6 * b];
@@ -1201,12 +1200,8 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         ngroup[b] = (gp.nseg[b] + kGradGroup - 1) / kGradGroup;
         if (fr.rects[4 * b + 2] <= 0) continue;
         groups = std::max(groups, ngroup[b]);
-        row_segs += static_cast<long long>(gp.nseg[b]) * fr.rects[4 * b + 2];
     }
-    // bands of image rows whose samples fit the workspace's bound
-    const long long row_bytes = row_segs * kGradSeg * static_cast<long long>(sizeof(float));
-    int band_h = static_cast<int>(
-        std::min<long long>(fr.H, row_bytes > 0 ? std::max(1LL, kGradBandBytes / row_bytes) : fr.H));
+    int band_h = fr.H;  // image rows per launch
     struct Band {
         long long segs = 0, groups = 0, px = 0;
     };
@@ -1233,9 +1228,10 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         return n;
     };
     // workspace: table copies, groups, samples, segments, counts (each part a
-    // multiple of 16 bytes from the start); where it cannot be had, smaller bands
+    // multiple of 16 bytes from the start); bands of rows where a view's samples do
+    // not fit its bound or it cannot be had
     auto part = [](long long n, size_t size) { return (static_cast<size_t>(n) * size + 15) & ~static_cast<size_t>(15); };
-    const size_t copies_bytes = part(static_cast<long long>(kGradCopies) * ctx->ntf * kGradEntry, sizeof(float));
+    const size_t copies_bytes = part(static_cast<long long>(kGradCopies) * (ctx->ntf + 1), sizeof(float4));
     size_t group_bytes, x_bytes, front_bytes;
     long long view_segs;
     for (;; band_h = (band_h + 1) / 2) {
@@ -1250,6 +1246,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         }
         group_bytes = part(most.groups, sizeof(float2));
         x_bytes = part(most.segs * kGradSeg, sizeof(float));
+        if (x_bytes > static_cast<size_t>(kGradBandBytes) && band_h > 1) continue;
         front_bytes = part(most.segs, sizeof(float));
         const size_t need = copies_bytes + group_bytes + x_bytes + front_bytes + part(most.px, sizeof(unsigned short));
         if (need <= ctx->grad_cap) break;

@@ -97,16 +97,16 @@ def test_storage_kinds_match_oracle(vr, storage, octets):
 
 
 def test_image_in_several_bands_matches_oracle(vr):
-    """Runs of up to 3700 samples over a 200 x 900 image: over 1 GB of samples per
-    368 rows, so three bands; the upstream gradient lives on pixels of all of
-    them, the band edges' rows among them. The ramp table has a slope everywhere
+    """Runs of up to 3700 samples over a 200 x 900 image: over 1 GB of samples, so
+    bands of 450 rows; the upstream gradient lives on pixels of both, the rows at
+    their edge among them. The ramp table has a slope everywhere
     and leaves the 3700 samples transparent enough for gradients in FP32's range."""
     rng = np.random.default_rng(8)
     vol, _ = _scene(rng, (64, 64, 64))
     tf = synth.ramp_tf(alpha_max=0.002)
     part = dict(kind="grid", grid=(1, 1, 1))
     cam = synth.orbit_camera(200, 900, 30.0, elevation_deg=20.0)
-    ys = np.concatenate([np.arange(330, 400), rng.integers(150, 750, 60)])
+    ys = np.concatenate([np.arange(330, 400), rng.integers(150, 750, 60), np.arange(440, 460)])
     pix = np.unique(np.stack([rng.integers(60, 140, ys.size), ys], axis=1), axis=0)
     g = rng.standard_normal((len(pix), 4)).astype(np.float32)
     G = np.zeros((900, 200, 4), np.float32)

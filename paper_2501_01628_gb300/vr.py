@@ -155,7 +155,12 @@ def _check(status: int, ctx=None, what: str = ""):
 def _stream(stream):
     if stream is None:
         import torch
-        if torch.cuda.is_available():
+        if torch.cuda.is_initialized() or torch.cuda.is_available():
+            # the current stream's handle without a torch.cuda.Stream object around it
+            # (0.3 us against 3.7 us; a small frame's calls take about 14)
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            if raw is not None:
+                return ctypes.c_void_p(raw(torch.cuda.current_device()))
             return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
         return ctypes.c_void_p(0)
     if isinstance(stream, int):

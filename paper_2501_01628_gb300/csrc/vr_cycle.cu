@@ -15,8 +15,16 @@ namespace {
 // where every ray visits every rank, restated for bricks on one GPU). No
 // partial images and no composite; early termination is global.
 // ---------------------------------------------------------------------------
+// Bound by the latency of a ray's chain of loads (a launch has one thread per
+// pixel, each with all its bricks' samples), so each ray keeps kWideSamples samples
+// in flight, at 8 blocks per SM. ms per frame, samples in pairs with the previous
+// cell's quads reused / four in flight: 512^3, 36 bricks, 1080p 0.581 / 0.544;
+// 256^3 at 1024^2 0.491 / 0.461, at 512^2 0.334 / 0.307, at 256^2 0.156 / 0.122;
+// 64^3 at 256^2 0.0214 / 0.0198. (Six or eight in flight: 0.269 and 0.230 at 512^2,
+// but 0.146 and 0.134 at 256^2, 0.481 and 0.476 at 1024^2.) The counting variant
+// keeps the pairs, whose quads' bounds it checks.
 template <typename S, bool COUNT, bool OPC>
-__global__ void __launch_bounds__(128) march_cycle_kernel(const __grid_constant__ MarchParams p, float4 *out)
+__global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_constant__ MarchParams p, float4 *out)
 {
     // pipelined frames: the next frame's kernel may start once every block of
     // this grid is running, and this grid's image store waits for the
@@ -36,8 +44,12 @@ __global__ void __launch_bounds__(128) march_cycle_kernel(const __grid_constant_
             continue;
         dev::OwnedRun run;
         dev::brick_run(p, B, ray, run);
-        dev::march_accumulate<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, C0, C1,
-                                             C2, T, executed, p.opc_ratio, p.count_error);
+        if constexpr (!COUNT)
+            dev::march_accumulate_wide<S, OPC, kWideSamples>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf,
+                                                             p.ert_T, C0, C1, C2, T, p.opc_ratio);
+        else
+            dev::march_accumulate<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, C0, C1,
+                                                 C2, T, executed, p.opc_ratio, p.count_error);
         if (T <= p.ert_T) break;
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -515,6 +515,87 @@ __device__ __forceinline__ void march_accumulate(const void *data, const BrickLa
     }
 }
 
+// The same run, same arithmetic and same results, U samples at a time: the
+// samples' quads are requested together, then their table entries, then they are
+// accumulated in order (past the run's end the last sample is requested again and
+// not accumulated). For launches that do not fill the chip, whose time is the
+// latency of one ray's chain of loads.
+template <typename S, bool OPC, int U>
+__device__ __forceinline__ void march_accumulate_wide(const void *data, const BrickLaunch &B, const OwnedRun &run,
+                                                      const float4 *tf, float tf_scale, float tf_bias, int ntf,
+                                                      float ert_T, float &C0, float &C1, float &C2, float &T,
+                                                      float opc_ratio)
+{
+    using Q = typename Quad<S>::type;
+    const Q *vox = static_cast<const Q *>(data) + B.base;
+    const unsigned nbx = static_cast<unsigned>(B.sx / 2), nby = static_cast<unsigned>(B.sy / 2);
+    const unsigned nbz = static_cast<unsigned>(B.hi[2] - B.lo[2] + 3) / 2;
+    const unsigned last = nbx * nby * nbz * 8u - 1u;
+    const unsigned ay = 4u * nbx, az = 4u * nbx * nby;
+    const unsigned c0 = 0u - (4u + ay + az) * kFloorBits;
+    const unsigned py = 2u - ay, pz = 4u - az, dz = 2u * az - 8u;
+    const float xmax = static_cast<float>(ntf - 1);
+    const uintptr_t tf_base = reinterpret_cast<uintptr_t>(tf) - static_cast<uintptr_t>(kFloorBits) * 32u;
+    auto floor_bits = [](float v, float &w) {
+        const float y = __fadd_rd(v, kFloorOffset);
+        w = v - (y - kFloorOffset);
+        return __float_as_uint(y);
+    };
+    for (int k = run.ka; k <= run.kb; k += U) {
+        float4 q0[U], q1[U];
+        float wx[U], wy[U], wz[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float h = static_cast<float>(min(k + u, run.kb)) + 0.5f;
+            const unsigned bx = floor_bits(fmaf(h, run.step[0], run.base[0]), wx[u]);
+            const unsigned by = floor_bits(fmaf(h, run.step[1], run.base[1]), wy[u]);
+            const unsigned bz = floor_bits(fmaf(h, run.step[2], run.base[2]), wz[u]);
+            unsigned c = bz * az + c0;
+            c = by * ay + c;
+            c = bx * 4u + c;
+            c = (bx & 1u) * (0u - 3u) + c;
+            c = (by & 1u) * py + c;
+            c = (bz & 1u) * pz + c;
+            const unsigned c1 = min(c + 4u + (bz & 1u) * dz, last);
+            c = min(c, last);
+            if constexpr (Quad<S>::octet) {
+                Quad<S>::load2(vox + c, q0[u], q1[u]);
+            } else {
+                q0[u] = Quad<S>::load(vox + c);
+                q1[u] = Quad<S>::load(vox + c1);
+            }
+        }
+        float4 e[U], d[U];
+        float w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float4 &a0 = q0[u], &a1 = q1[u];
+            const float c00 = fmaf(wx[u], a0.y - a0.x, a0.x), c10 = fmaf(wx[u], a0.w - a0.z, a0.z);
+            const float c01 = fmaf(wx[u], a1.y - a1.x, a1.x), c11 = fmaf(wx[u], a1.w - a1.z, a1.z);
+            const float c0_ = fmaf(wy[u], c10 - c00, c00), c1_ = fmaf(wy[u], c11 - c01, c01);
+            const float x = fminf(fmaxf(fmaf(fmaf(wz[u], c1_ - c0_, c0_), tf_scale, tf_bias), 0.0f), xmax);
+            ldg_v8(reinterpret_cast<const float4 *>(tf_base + static_cast<uintptr_t>(floor_bits(x, w[u])) * 32u), e[u],
+                   d[u]);
+        }
+        bool ended = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (ended || k + u > run.kb) continue;
+            const float r = fmaf(w[u], d[u].x, e[u].x), g = fmaf(w[u], d[u].y, e[u].y);
+            const float b = fmaf(w[u], d[u].z, e[u].z);
+            float al = fmaf(w[u], d[u].w, e[u].w);
+            if (OPC) al = -expm1f(opc_ratio * log1pf(-al));
+            const float ta = T * al;
+            C0 = fmaf(ta, r, C0);
+            C1 = fmaf(ta, g, C1);
+            C2 = fmaf(ta, b, C2);
+            T = T - ta;
+            ended = T <= ert_T;
+        }
+        if (ended) break;
+    }
+}
+
 // One brick's partial from a fresh state: (C, 1 - T).
 template <typename S, bool COUNT, bool OPC = false>
 __device__ __forceinline__ float4 march_run(const void *data, const BrickLaunch &B, const OwnedRun &run,

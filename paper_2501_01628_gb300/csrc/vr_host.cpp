@@ -528,6 +528,18 @@ void timing_end(vr_ctx ctx, int idx, cudaStream_t s)
     if (idx >= 0) cudaEventRecord(ctx->timed[idx].b, s);
 }
 
+// The march with several samples of a ray in flight (same image) for launches of
+// at most six blocks per multiprocessor, which do not fill it at either kernel's
+// registers (64 and 56: 8 and 9 blocks): their time is one ray's latency. us per
+// frame pairs / wide, pipelined and in sequence: 24 blocks 8.2 / 5.3 and 26.7 / 20.5;
+// 520 blocks (64^3 at 256^2) 13.6 / 12.7 and 24.7 / 24.6; 538 blocks, 128^3 26.5 / 25.8
+// and 53.4 / 45.2, 256^3 92.0 / 78.8 and 211 / 141; 943 blocks 119 / 107 and 221 / 160.
+// Above, either may win by view (1075 blocks 491 / 502 and 800 / 704, 1145 blocks 39.6 /
+// 39.2 and 58.4 / 61.5, 2705 blocks 330 / 304, 3721 blocks 344 / 357), and full launches,
+// bound by the L1 that the pairs' reuse of the previous cell saves, lose 2 to 6%.
+constexpr int kWideBlocks = 6;
+bool wide_march(vr_ctx ctx, int blocks) { return blocks <= kWideBlocks * ctx->sms; }
+
 vr_status march(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, cudaStream_t s, bool after_composite = false,
                 const PoolSync *sync = nullptr)
 {
@@ -557,7 +569,7 @@ vr_status march(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, cudaStream_t s, bool 
         }
         VR_LAUNCH(ctx, launch_march_staged(mp, sb, s));
     } else {
-        VR_LAUNCH(ctx, launch_march(mp, vol->kind(), s, after_composite));
+        VR_LAUNCH(ctx, launch_march(mp, vol->kind(), s, after_composite, wide_march(ctx, mp.n_items)));
     }
     timing_end(ctx, t, s);
     return VR_OK;

@@ -204,12 +204,16 @@ struct StagedBricks {
     int sxp[kMaxBricks];          // padded row length (elements)
 };
 
+constexpr int kWideSamples = 4;  // samples in flight per ray of a wide march (dev::march_accumulate_wide)
+
 // Launchers (vr_kernels.cu). They return the launch's cudaError_t.
 // `kind` is a StorageKind.
 cudaError_t launch_pack(const PackParams &p, int kind, cudaStream_t s);
 // after_composite: launch as a programmatic dependent of the preceding kernel
 // (the previous pipelined frame's composite); see march_kernel.
-cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool after_composite = false);
+// wide: the march for launches that do not fill the chip (same image).
+cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool after_composite = false,
+                         bool wide = false);
 // after_frame: launch as a programmatic dependent of the preceding kernel (the
 // previous pipelined frame); see march_cycle_kernel.
 cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cudaStream_t s, bool after_frame = false);

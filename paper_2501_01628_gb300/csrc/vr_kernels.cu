@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constan
 // function is read as (T[i], T[i+1]-T[i]) pairs (the last difference is 0)
 // through L1: one cached copy per SM instead of one shared-memory copy per block.
 // ---------------------------------------------------------------------------
-template <typename S, bool COUNT, bool OPC>
-__global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ MarchParams p)
+template <typename S, bool COUNT, bool OPC, bool WIDE>
+__device__ __forceinline__ void march_block(const MarchParams &p)
 {
     // the composite launched after this march may start once every block of
     // this grid is running; it reads the masks and partials only after this
@@ -168,9 +168,16 @@ __global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ Marc
     unsigned long long executed = 0;
     dev::OwnedRun run;
     dev::owned_run(p, B, px, py, run);
-    const float4 c =
-        dev::march_run<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, executed, p.opc_ratio,
-                                      p.count_error);
+    float4 c;
+    if constexpr (WIDE) {
+        float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
+        dev::march_accumulate_wide<S, OPC, kWideSamples>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, C0,
+                                                         C1, C2, T, p.opc_ratio);
+        c = make_float4(C0, C1, C2, 1.0f - T);
+    } else {
+        c = dev::march_run<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, executed,
+                                          p.opc_ratio, p.count_error);
+    }
     // the composite reads the partial next: keep it in L2 ahead of the streamed bricks
     float4 *dst = p.partials + B.poff + static_cast<long long>(ry) * B.rect[2] + rx;
     if (!dev::pool_ready(p.pool_done, p.pool, p.pool_frame, p.count_error)) return;
@@ -180,6 +187,20 @@ __global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ Marc
                  "f"(c.z), "f"(c.w), "l"(policy)
                  : "memory");
     if (COUNT && executed) atomicAdd(p.sample_counter, executed);
+}
+
+template <typename S, bool COUNT, bool OPC>
+__global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ MarchParams p)
+{
+    march_block<S, COUNT, OPC, false>(p);
+}
+
+// For launches that do not fill the chip (wide_march in vr_host.cpp has the rule
+// and its figures).
+template <typename S, bool OPC>
+__global__ void __launch_bounds__(128) march_wide_kernel(const __grid_constant__ MarchParams p)
+{
+    march_block<S, false, OPC, true>(p);
 }
 
 }  // namespace
@@ -201,7 +222,7 @@ cudaError_t launch_pack(const PackParams &p, int kind, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool after_composite)
+cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool after_composite, bool wide)
 {
     if (p.n_items + p.mask_blocks <= 0) return cudaSuccess;
     const int grid = p.n_items + p.mask_blocks;
@@ -217,7 +238,9 @@ cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool af
     cfg.attrs = attr;
     cfg.numAttrs = after_composite ? 1 : 0;
 #define VR_MARCH(T)                                                                                     \
-    (opc ? (count ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, true>, p)                       \
+    (wide && !count ? (opc ? cudaLaunchKernelEx(&cfg, march_wide_kernel<T, true>, p)               \
+                           : cudaLaunchKernelEx(&cfg, march_wide_kernel<T, false>, p))             \
+     : opc ? (count ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, true>, p)                       \
                   : cudaLaunchKernelEx(&cfg, march_kernel<T, false, true>, p))                     \
          : (count ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, false>, p)                      \
                   : cudaLaunchKernelEx(&cfg, march_kernel<T, false, false>, p)))

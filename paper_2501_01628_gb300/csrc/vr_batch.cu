@@ -43,7 +43,7 @@ __device__ __forceinline__ bool wait_at_least(const int *addr, int target, int l
     return false;
 }
 
-template <typename S, bool OPC>
+template <typename S, int OPC>
 __global__ void __launch_bounds__(128, 9) batch_kernel(const __grid_constant__ BatchParams p)
 {
     __shared__ long long s_item;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(128, 9) batch_kernel(const __grid_constant__ B
                 const float2 sb = p.vol_tf[v];
                 part[B.poff + static_cast<long long>(ry) * B.rect[2] + rx] =
                     dev::march_run<S, false, OPC>(p.vol_data[v], B, run, p.tf, sb.x, sb.y, p.ntf, p.ert_T, unused,
-                                                  p.opc_ratio);
+                                                  p.opc);
             }
             __threadfence();  // every writer publishes its partial before the count moves
             __syncthreads();
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(128, 9) batch_kernel(const __grid_constant__ B
     }
 }
 
-template <typename S, bool OPC>
+template <typename S, int OPC>
 cudaError_t launch_batch_t(const BatchParams &p, int blocks, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -214,7 +214,10 @@ cudaError_t launch_batch_t(const BatchParams &p, int blocks, cudaStream_t s)
 template <typename S>
 cudaError_t launch_batch_s(const BatchParams &p, int blocks, cudaStream_t s)
 {
-    return p.opc_ratio != 1.0f ? launch_batch_t<S, true>(p, blocks, s) : launch_batch_t<S, false>(p, blocks, s);
+    const int opc = opacity_kind(p.opc);
+    return opc == kOpacitySeries    ? launch_batch_t<S, kOpacitySeries>(p, blocks, s)
+           : opc == kOpacityGeneral ? launch_batch_t<S, kOpacityGeneral>(p, blocks, s)
+                                    : launch_batch_t<S, kOpacityOff>(p, blocks, s);
 }
 
 cudaError_t launch_batch(const BatchParams &p, int kind, int blocks, cudaStream_t s)
@@ -229,23 +232,28 @@ cudaError_t launch_batch(const BatchParams &p, int kind, int blocks, cudaStream_
     }
 }
 
+// What fits of every variant: a batch keeps its plan when the correction changes.
+template <typename S>
+int batch_fits()
+{
+    int n[3] = {};
+    const bool ok =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[0], batch_kernel<S, kOpacityOff>, 128, 0) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[1], batch_kernel<S, kOpacityGeneral>, 128, 0) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[2], batch_kernel<S, kOpacitySeries>, 128, 0) == cudaSuccess;
+    return ok ? std::min(n[0], std::min(n[1], n[2])) : 0;
+}
+
 int batch_max_blocks_per_sm(int kind)
 {
-    int n = 0;
-    cudaError_t e = cudaErrorInvalidValue;
     switch (kind) {
-    case kStoreF32: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<float, true>, 128, 0); break;
-    case kStoreBF16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<__nv_bfloat16, true>, 128, 0); break;
-    case kStoreF16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<__half, true>, 128, 0); break;
-    case kStoreBF16Oct:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<dev::Octet<__nv_bfloat16>, true>, 128, 0);
-        break;
-    case kStoreF16Oct:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<dev::Octet<__half>, true>, 128, 0);
-        break;
-    default: break;
+    case kStoreF32: return batch_fits<float>();
+    case kStoreBF16: return batch_fits<__nv_bfloat16>();
+    case kStoreF16: return batch_fits<__half>();
+    case kStoreBF16Oct: return batch_fits<dev::Octet<__nv_bfloat16>>();
+    case kStoreF16Oct: return batch_fits<dev::Octet<__half>>();
+    default: return 0;
     }
-    return e == cudaSuccess ? n : 0;
 }
 
 }  // namespace vr
@@ -468,7 +476,8 @@ vr_status build(vr_batch b, int pw, int bps, int mode)
     p.tf = ctx->d_tf;
     p.ntf = ctx->ntf;
     p.ert_T = ctx->ert_alpha < 1.0f ? static_cast<float>(1.0 - static_cast<double>(ctx->ert_alpha)) : -1.0f;
-    p.opc_ratio = ctx->opc_ref > 0.0f ? static_cast<float>(static_cast<double>(ctx->step) / ctx->opc_ref) : 1.0f;
+    p.opc = opacity_step(ctx->opc_ref > 0.0f ? static_cast<float>(static_cast<double>(ctx->step) / ctx->opc_ref) : 1.0f,
+                          ctx->tf_alpha_max);
     p.ring = b->d_ring;
     p.slot_px = unit_px;
     p.slots = slots;

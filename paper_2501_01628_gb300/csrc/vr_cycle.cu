@@ -23,7 +23,7 @@ namespace {
 // 64^3 at 256^2 0.0214 / 0.0198. (Six or eight in flight: 0.269 and 0.230 at 512^2,
 // but 0.146 and 0.134 at 256^2, 0.481 and 0.476 at 1024^2.) The counting variant
 // keeps the pairs, whose quads' bounds it checks.
-template <typename S, bool COUNT, bool OPC>
+template <typename S, bool COUNT, int OPC>
 __global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_constant__ MarchParams p, float4 *out)
 {
     // pipelined frames: the next frame's kernel may start once every block of
@@ -46,10 +46,10 @@ __global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_consta
         dev::brick_run(p, B, ray, run);
         if constexpr (!COUNT)
             dev::march_accumulate_wide<S, OPC, kWideSamples>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf,
-                                                             p.ert_T, C0, C1, C2, T, p.opc_ratio);
+                                                             p.ert_T, C0, C1, C2, T, p.opc);
         else
             dev::march_accumulate<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, C0, C1,
-                                                 C2, T, executed, p.opc_ratio, p.count_error);
+                                                 C2, T, executed, p.opc, p.count_error);
         if (T <= p.ert_T) break;
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -64,7 +64,7 @@ cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cuda
     if (p.W <= 0 || p.H <= 0) return cudaSuccess;
     const dim3 grid((p.W + p.tile_w - 1) / p.tile_w, (p.H + p.tile_h - 1) / p.tile_h);
     const bool count = p.sample_counter != nullptr;
-    const bool opc = p.opc_ratio != 1.0f;
+    const bool opc = opacity_kind(p.opc) != kOpacityOff;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -74,11 +74,11 @@ cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cuda
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = after_frame ? 1 : 0;
-#define VR_CYCLE(T)                                                                                    \
-    (opc ? (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, true>, p, out)                \
-                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, true>, p, out))              \
-         : (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, false>, p, out)               \
-                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, false>, p, out)))
+#define VR_CYCLE(T)                                                                              \
+    (opc ? (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, kOpacitySeries>, p, out)    \
+                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, kOpacitySeries>, p, out))  \
+         : (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, kOpacityOff>, p, out)       \
+                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, kOpacityOff>, p, out)))
     cudaError_t e = cudaErrorInvalidValue;
     switch (kind) {
     case kStoreF32: e = VR_CYCLE(float); break;

@@ -480,7 +480,8 @@ vr_status prepare_frame(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, MarchParams &
     mp.dt = static_cast<float>(dt);
     mp.inv_dt = static_cast<float>(1.0 / dt);
     mp.ert_T = ctx->ert_alpha < 1.0f ? static_cast<float>(1.0 - static_cast<double>(ctx->ert_alpha)) : -1.0f;
-    mp.opc_ratio = ctx->opc_ref > 0.0f ? static_cast<float>(static_cast<double>(ctx->step) / ctx->opc_ref) : 1.0f;
+    mp.opc = opacity_step(ctx->opc_ref > 0.0f ? static_cast<float>(static_cast<double>(ctx->step) / ctx->opc_ref) : 1.0f,
+                           ctx->tf_alpha_max);
     {
         const double scale = (ctx->ntf - 1) / (static_cast<double>(ctx->vmax) - ctx->vmin);
         mp.tf_scale = static_cast<float>(scale);
@@ -1401,8 +1402,9 @@ vr_status table_room(vr_ctx ctx, const float *rgba, int n, float vmin, float vma
     return VR_OK;
 }
 
-void table_set(vr_ctx ctx, int n, float vmin, float vmax)
+void table_set(vr_ctx ctx, int n, float vmin, float vmax, float alpha_max)
 {
+    ctx->tf_alpha_max = alpha_max;
     ctx->ntf = n;
     ctx->vmin = vmin;
     ctx->vmax = vmax;
@@ -1418,6 +1420,7 @@ vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float v
     if (st != VR_OK) return st;
     // device table: (T[i], T[i+1] - T[i]) pairs in float32, last difference 0
     std::vector<float> t(4 * static_cast<size_t>(n)), pairs(8 * static_cast<size_t>(n));
+    float alpha_max = 0.0f;
     if (on_device)
         VR_CUDA(ctx, cudaMemcpy(t.data(), rgba, t.size() * sizeof(float), cudaMemcpyDeviceToHost));
     else
@@ -1428,10 +1431,11 @@ vr_status vr_set_transfer_function(vr_ctx ctx, const float *rgba, int n, float v
             const float b = i + 1 < n ? t[4 * (i + 1) + c] : a;
             pairs[8 * i + c] = a;
             pairs[8 * i + 4 + c] = b - a;
+            if (c == 3 && !(std::fabs(a) <= alpha_max)) alpha_max = std::isnan(a) ? INFINITY : std::fabs(a);
         }
     ctx->input_seq++;  // a pipelined march must not read the table across this upload
     VR_CUDA(ctx, cudaMemcpy(ctx->d_tf, pairs.data(), pairs.size() * sizeof(float), cudaMemcpyHostToDevice));
-    table_set(ctx, n, vmin, vmax);
+    table_set(ctx, n, vmin, vmax, alpha_max);
     return VR_OK;
 }
 
@@ -1447,7 +1451,7 @@ vr_status vr_set_transfer_function_async(vr_ctx ctx, const float *rgba_dev, int 
     ctx->input_seq++;  // a pipelined march must not read the table across this kernel
     VR_LAUNCH(ctx, launch_table_pairs(reinterpret_cast<const float4 *>(rgba_dev), n, ctx->d_tf,
                                       static_cast<cudaStream_t>(stream)));
-    table_set(ctx, n, vmin, vmax);
+    table_set(ctx, n, vmin, vmax, INFINITY);
     return VR_OK;
 }
 

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constan
 // function is read as (T[i], T[i+1]-T[i]) pairs (the last difference is 0)
 // through L1: one cached copy per SM instead of one shared-memory copy per block.
 // ---------------------------------------------------------------------------
-template <typename S, bool COUNT, bool OPC, bool WIDE>
+template <typename S, bool COUNT, int OPC, bool WIDE>
 __device__ __forceinline__ void march_block(const MarchParams &p)
 {
     // the composite launched after this march may start once every block of
@@ -172,11 +172,11 @@ __device__ __forceinline__ void march_block(const MarchParams &p)
     if constexpr (WIDE) {
         float C0 = 0.f, C1 = 0.f, C2 = 0.f, T = 1.f;
         dev::march_accumulate_wide<S, OPC, kWideSamples>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, C0,
-                                                         C1, C2, T, p.opc_ratio);
+                                                         C1, C2, T, p.opc);
         c = make_float4(C0, C1, C2, 1.0f - T);
     } else {
         c = dev::march_run<S, COUNT, OPC>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf, p.ert_T, executed,
-                                          p.opc_ratio, p.count_error);
+                                          p.opc, p.count_error);
     }
     // the composite reads the partial next: keep it in L2 ahead of the streamed bricks
     float4 *dst = p.partials + B.poff + static_cast<long long>(ry) * B.rect[2] + rx;
@@ -189,7 +189,7 @@ __device__ __forceinline__ void march_block(const MarchParams &p)
     if (COUNT && executed) atomicAdd(p.sample_counter, executed);
 }
 
-template <typename S, bool COUNT, bool OPC>
+template <typename S, bool COUNT, int OPC>
 __global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ MarchParams p)
 {
     march_block<S, COUNT, OPC, false>(p);
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(128) march_kernel(const __grid_constant__ Marc
 
 // For launches that do not fill the chip (wide_march in vr_host.cpp has the rule
 // and its figures).
-template <typename S, bool OPC>
+template <typename S, int OPC>
 __global__ void __launch_bounds__(128) march_wide_kernel(const __grid_constant__ MarchParams p)
 {
     march_block<S, false, OPC, true>(p);
@@ -227,7 +227,7 @@ cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool af
     if (p.n_items + p.mask_blocks <= 0) return cudaSuccess;
     const int grid = p.n_items + p.mask_blocks;
     const bool count = p.sample_counter != nullptr;
-    const bool opc = p.opc_ratio != 1.0f;
+    const int opc = opacity_kind(p.opc);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -237,13 +237,14 @@ cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool af
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = after_composite ? 1 : 0;
-#define VR_MARCH(T)                                                                                     \
-    (wide && !count ? (opc ? cudaLaunchKernelEx(&cfg, march_wide_kernel<T, true>, p)               \
-                           : cudaLaunchKernelEx(&cfg, march_wide_kernel<T, false>, p))             \
-     : opc ? (count ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, true>, p)                       \
-                  : cudaLaunchKernelEx(&cfg, march_kernel<T, false, true>, p))                     \
-         : (count ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, false>, p)                      \
-                  : cudaLaunchKernelEx(&cfg, march_kernel<T, false, false>, p)))
+#define VR_MARCH(T)                                                                                      \
+    (wide && !count ? (opc ? cudaLaunchKernelEx(&cfg, march_wide_kernel<T, kOpacitySeries>, p)           \
+                           : cudaLaunchKernelEx(&cfg, march_wide_kernel<T, kOpacityOff>, p))             \
+     : count ? (opc ? cudaLaunchKernelEx(&cfg, march_kernel<T, true, kOpacitySeries>, p)                 \
+                    : cudaLaunchKernelEx(&cfg, march_kernel<T, true, kOpacityOff>, p))                   \
+     : opc == kOpacitySeries    ? cudaLaunchKernelEx(&cfg, march_kernel<T, false, kOpacitySeries>, p)    \
+       : opc == kOpacityGeneral ? cudaLaunchKernelEx(&cfg, march_kernel<T, false, kOpacityGeneral>, p)   \
+                                : cudaLaunchKernelEx(&cfg, march_kernel<T, false, kOpacityOff>, p))
     cudaError_t e = cudaErrorInvalidValue;
     switch (kind) {
     case kStoreF32: e = VR_MARCH(float); break;

@@ -81,7 +81,7 @@ __device__ int locate(const MeshNode *nodes, const float4 *rec, float qx, float 
 
 // A mask block writes one tile mask per thread.
 static_assert(kMaskThreads == 128, "mask blocks are march blocks");
-template <bool COUNT, bool OPC>
+template <bool COUNT, int OPC>
 __global__ void __launch_bounds__(128, 8) march_mesh_kernel(const __grid_constant__ MeshParams P)
 {
     const MarchParams &p = P.m;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(128, 8) march_mesh_kernel(const __grid_constan
             };
             auto accumulate = [&](float w, const float4 &e0, const float4 &de) {
                 float al = fmaf(w, de.w, e0.w);
-                if (OPC) al = -expm1f(p.opc_ratio * log1pf(-al));
+                if (OPC) al = dev::corrected_opacity<OPC>(al, p.opc);
                 const float ta = T * al;
                 C0 = fmaf(ta, fmaf(w, de.x, e0.x), C0);
                 C1 = fmaf(ta, fmaf(w, de.y, e0.y), C1);
@@ -277,7 +277,8 @@ cudaError_t launch_march_mesh(const MeshParams &p, cudaStream_t s, bool after_fr
 {
     const int grid = p.m.n_items + p.m.mask_blocks;
     if (grid <= 0) return cudaSuccess;
-    const bool count = p.m.sample_counter != nullptr, opc = p.m.opc_ratio != 1.0f;
+    const bool count = p.m.sample_counter != nullptr;
+    const int opc = opacity_kind(p.m.opc);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -287,10 +288,11 @@ cudaError_t launch_march_mesh(const MeshParams &p, cudaStream_t s, bool after_fr
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = after_frame ? 1 : 0;
-    if (count) return opc ? cudaLaunchKernelEx(&cfg, march_mesh_kernel<true, true>, p)
-                          : cudaLaunchKernelEx(&cfg, march_mesh_kernel<true, false>, p);
-    return opc ? cudaLaunchKernelEx(&cfg, march_mesh_kernel<false, true>, p)
-               : cudaLaunchKernelEx(&cfg, march_mesh_kernel<false, false>, p);
+    if (count) return opc ? cudaLaunchKernelEx(&cfg, march_mesh_kernel<true, kOpacitySeries>, p)
+                          : cudaLaunchKernelEx(&cfg, march_mesh_kernel<true, kOpacityOff>, p);
+    return opc == kOpacitySeries    ? cudaLaunchKernelEx(&cfg, march_mesh_kernel<false, kOpacitySeries>, p)
+           : opc == kOpacityGeneral ? cudaLaunchKernelEx(&cfg, march_mesh_kernel<false, kOpacityGeneral>, p)
+                                    : cudaLaunchKernelEx(&cfg, march_mesh_kernel<false, kOpacityOff>, p);
 }
 
 }  // namespace vr

@@ -92,6 +92,7 @@ struct vr_ctx_s {
     int ntf = 0;
     int tf_cap = 0;
     float vmin = 0.f, vmax = 1.f;
+    float tf_alpha_max = INFINITY;  // largest |opacity| in the table (infinity: set on the device)
     bool has_tf = false;
     vr_camera cam{};
     bool has_cam = false;

@@ -82,7 +82,7 @@ struct Slab {
 
 constexpr int kWaitLimit = 1 << 22;
 
-template <bool COUNT, bool OPC>
+template <bool COUNT, int OPC>
 __global__ void __launch_bounds__(128) march_staged_kernel(const __grid_constant__ MarchParams p,
                                                            const __grid_constant__ StagedBricks sb)
 {
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(128) march_staged_kernel(const __grid_constant
                                 e0, de);
                     const float r = fmaf(w, de.x, e0.x), g = fmaf(w, de.y, e0.y), bb = fmaf(w, de.z, e0.z);
                     float al = fmaf(w, de.w, e0.w);
-                    if (OPC) al = -expm1f(p.opc_ratio * log1pf(-al));
+                    if (OPC) al = dev::corrected_opacity<OPC>(al, p.opc);
                     const float ta = T * al;
                     C0 = fmaf(ta, r, C0);
                     C1 = fmaf(ta, g, C1);
@@ -400,13 +400,13 @@ cudaError_t launch_march_staged(const MarchParams &p, const StagedBricks &sb, cu
     if (grid <= 0) return cudaSuccess;
     constexpr size_t smem = 2 * kStageCap * sizeof(float);
     const bool count = p.sample_counter != nullptr;
-    const bool opc = p.opc_ratio != 1.0f;
+    const bool opc = opacity_kind(p.opc) != kOpacityOff;
     if (opc) {
-        if (count) march_staged_kernel<true, true><<<grid, 128, smem, s>>>(p, sb);
-        else march_staged_kernel<false, true><<<grid, 128, smem, s>>>(p, sb);
+        if (count) march_staged_kernel<true, kOpacitySeries><<<grid, 128, smem, s>>>(p, sb);
+        else march_staged_kernel<false, kOpacitySeries><<<grid, 128, smem, s>>>(p, sb);
     } else {
-        if (count) march_staged_kernel<true, false><<<grid, 128, smem, s>>>(p, sb);
-        else march_staged_kernel<false, false><<<grid, 128, smem, s>>>(p, sb);
+        if (count) march_staged_kernel<true, kOpacityOff><<<grid, 128, smem, s>>>(p, sb);
+        else march_staged_kernel<false, kOpacityOff><<<grid, 128, smem, s>>>(p, sb);
     }
     return cudaGetLastError();
 }

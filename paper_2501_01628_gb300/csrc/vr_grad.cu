@@ -66,12 +66,21 @@ struct GradCell {
         c = (by & 1u) * G.py + c;
         return (bz & 1u) * G.pz + c;
     }
-    __device__ __forceinline__ unsigned quad(const GradBrick &G) const { return min(place(G), G.last); }
     __device__ __forceinline__ void quads(const GradBrick &G, unsigned &c, unsigned &c1) const
     {
         const unsigned at = place(G);
         c = min(at, G.last);
         c1 = min(at + 4u + (bz & 1u) * G.dz, G.last);
+    }
+    // the same two by the parity of their plane
+    __device__ __forceinline__ void planes(const GradBrick &G, unsigned &even, unsigned &odd) const
+    {
+        unsigned c = by * G.ay + G.c0;
+        c = bx * 4u + c;
+        c = (bx & 1u) * (0u - 3u) + c;
+        c = (by & 1u) * G.py + c;
+        even = min(((bz + 1u) & ~1u) * G.az + c, G.last);
+        odd = min((bz & ~1u) * G.az + c + 4u, G.last);
     }
 };
 
@@ -304,11 +313,13 @@ __device__ __forceinline__ void red_v4(float4 *dst, const float (&v)[4])
 // grad_voxels_kernel then adds them to the voxels), or with one reduction per
 // corner on the original volume's indexing (halo copies alias their neighbours'
 // voxels).
-// Bound by issue (63% of slots) at 23 of 32 lanes, then by the reductions on their
-// way to L2 (35% of its rate): 0.37 ms for a 512^2 view of a 256^3 volume (0.46 with
-// both entries and both planes added at every change; one thread per run with
-// shared-memory table gradients and three samplings took 2.1 ms). 4 and 6 blocks
-// per SM measured the same and 4% more.
+// Bound by issue (64% of slots) at 26.5 of 32 lanes, then by the reductions on their
+// way to L2 (39% of its rate): 0.32 ms for a 512^2 view of a 256^3 volume. A whole backward of 512^2 views of a 256^3 volume: 0.703 ms
+// with the sums by parity of their place, 0.743 ms with them moved between lower and
+// upper (0.37 ms here); one thread per run with shared-memory table gradients and
+// three samplings took 2.1 ms. 4 and 6 blocks per SM: 0.718 and 0.743 ms; segments of 4
+// samples 0.76, groups of 6 and 16 segments 0.718 and 0.701 (0.21 against 0.16 for a 256^2
+// view of 128^3).
 template <bool QUADS>
 __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_constant__ GradParams p)
 {
@@ -327,65 +338,61 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
     float4 *copy = reinterpret_cast<float4 *>(p.tf_copies) + static_cast<long long>(which) * (m.ntf + 1);
     const bool voxels = QUADS || p.grad_vol;
     float4 *gquads = QUADS ? p.grad_quads + B.base : nullptr;
-    // the cell being summed: quad index of its lower plane, floors (0: no cell)
-    unsigned cur_c = 0, cur_x = 0, cur_y = 0, cur_z = 0;
-    float lower[4], upper[4];
-    int cur_ti = -4;  // the table interval being summed (negative: none)
-    float at0[4], at1[4];
+    // Sums in registers by the parity of their place: of the two table entries of an
+    // interval, and of the two planes of a cell, one is even and one is odd, so that
+    // what the next sample shares stays where it is and what it leaves behind goes.
+    int cur_e = -1, cur_o = -1;  // entries being summed (negative: none)
+    float tab_e[4], tab_o[4], pl_e[4], pl_o[4];
+    unsigned quad_e = ~0u, quad_o = ~0u;          // QUADS: quads of the planes (~0: none)
+    unsigned cur_x = 0, cur_y = 0, cur_z = 0;     // else: the cell's floors (0: no cell)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) lower[c] = upper[c] = at0[c] = at1[c] = 0.0f;
-    // on to interval ti: an entry that the next interval shares stays in registers
-    auto next_interval = [&](int ti) {
-        const bool up = ti - cur_ti == 1, down = cur_ti - ti == 1;
-        if (cur_ti >= 0) {
-            if (!down) red_v4(copy + cur_ti, at0);
-            if (!up) red_v4(copy + cur_ti + 1, at1);
-        }
+    for (int c = 0; c < 4; ++c) tab_e[c] = tab_o[c] = pl_e[c] = pl_o[c] = 0.0f;
+    auto leave = [&](float4 *dst, bool any, float (&sum)[4]) {
+        if (any) red_v4(dst, sum);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float lo = at0[c], hi = at1[c];
-            at0[c] = up ? hi : 0.0f;
-            at1[c] = down ? lo : 0.0f;
-        }
-        cur_ti = ti;
+        for (int c = 0; c < 4; ++c) sum[c] = 0.0f;
     };
-    // on to cell q, likewise for the plane that a step along z shares
+    auto leave_cell = [&]() {  // the eight corners of (cur_x, cur_y, cur_z) into the voxels
+        const int i = static_cast<int>(cur_x - dev::kFloorBits), j = static_cast<int>(cur_y - dev::kFloorBits),
+                  k = static_cast<int>(cur_z - dev::kFloorBits);
+        const int gx0 = min(max(B.lo[0] - 1 + i, 0), p.N[0] - 1), gx1 = min(max(B.lo[0] + i, 0), p.N[0] - 1);
+        const int gy0 = min(max(B.lo[1] - 1 + j, 0), p.N[1] - 1), gy1 = min(max(B.lo[1] + j, 0), p.N[1] - 1);
+        const int ge = min(max(B.lo[2] - 1 + ((k + 1) & ~1), 0), p.N[2] - 1);
+        const int go = min(max(B.lo[2] - 1 + (k | 1), 0), p.N[2] - 1);
+        const long long nx = p.N[0], nxy = static_cast<long long>(p.N[0]) * p.N[1];
+        float *gv = p.grad_vol;
+        atomicAdd(gv + ge * nxy + gy0 * nx + gx0, pl_e[0]);
+        atomicAdd(gv + ge * nxy + gy0 * nx + gx1, pl_e[1]);
+        atomicAdd(gv + ge * nxy + gy1 * nx + gx0, pl_e[2]);
+        atomicAdd(gv + ge * nxy + gy1 * nx + gx1, pl_e[3]);
+        atomicAdd(gv + go * nxy + gy0 * nx + gx0, pl_o[0]);
+        atomicAdd(gv + go * nxy + gy0 * nx + gx1, pl_o[1]);
+        atomicAdd(gv + go * nxy + gy1 * nx + gx0, pl_o[2]);
+        atomicAdd(gv + go * nxy + gy1 * nx + gx1, pl_o[3]);
+    };
+    // on to cell q
     auto next_cell = [&](const GradCell &q) {
-        const bool column = q.bx == cur_x && q.by == cur_y;
-        const bool up = QUADS && column && q.bz - cur_z == 1u, down = QUADS && column && cur_z - q.bz == 1u;
-        if (cur_x != 0) {
-            if constexpr (QUADS) {
-                if (!down) red_v4(gquads + cur_c, lower);
-                if (!up) red_v4(gquads + min(cur_c + 4u + (cur_z & 1u) * G.dz, G.last), upper);
-            } else {
-                const int i = static_cast<int>(cur_x - dev::kFloorBits), j = static_cast<int>(cur_y - dev::kFloorBits),
-                          k = static_cast<int>(cur_z - dev::kFloorBits);
-                const int gx0 = min(max(B.lo[0] - 1 + i, 0), p.N[0] - 1), gx1 = min(max(B.lo[0] + i, 0), p.N[0] - 1);
-                const int gy0 = min(max(B.lo[1] - 1 + j, 0), p.N[1] - 1), gy1 = min(max(B.lo[1] + j, 0), p.N[1] - 1);
-                const int gz0 = min(max(B.lo[2] - 1 + k, 0), p.N[2] - 1), gz1 = min(max(B.lo[2] + k, 0), p.N[2] - 1);
-                const long long nx = p.N[0], nxy = static_cast<long long>(p.N[0]) * p.N[1];
-                float *gv = p.grad_vol;
-                atomicAdd(gv + gz0 * nxy + gy0 * nx + gx0, lower[0]);
-                atomicAdd(gv + gz0 * nxy + gy0 * nx + gx1, lower[1]);
-                atomicAdd(gv + gz0 * nxy + gy1 * nx + gx0, lower[2]);
-                atomicAdd(gv + gz0 * nxy + gy1 * nx + gx1, lower[3]);
-                atomicAdd(gv + gz1 * nxy + gy0 * nx + gx0, upper[0]);
-                atomicAdd(gv + gz1 * nxy + gy0 * nx + gx1, upper[1]);
-                atomicAdd(gv + gz1 * nxy + gy1 * nx + gx0, upper[2]);
-                atomicAdd(gv + gz1 * nxy + gy1 * nx + gx1, upper[3]);
+        if constexpr (QUADS) {
+            unsigned e, o;
+            q.planes(G, e, o);
+            if (e != quad_e) {
+                leave(gquads + quad_e, quad_e != ~0u, pl_e);
+                quad_e = e;
             }
-        }
+            if (o != quad_o) {
+                leave(gquads + quad_o, quad_o != ~0u, pl_o);
+                quad_o = o;
+            }
+        } else if (q.bx != cur_x || q.by != cur_y || q.bz != cur_z) {
+            if (cur_x != 0) leave_cell();
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float lo = lower[c], hi = upper[c];
-            lower[c] = up ? hi : 0.0f;
-            upper[c] = down ? lo : 0.0f;
+            for (int c = 0; c < 4; ++c) pl_e[c] = pl_o[c] = 0.0f;
+            cur_x = q.bx;
+            cur_y = q.by;
+            cur_z = q.bz;
         }
-        cur_x = q.bx;
-        cur_y = q.by;
-        cur_z = q.bz;
-        if constexpr (QUADS) cur_c = q.quad(G);
     };
+    const unsigned area = static_cast<unsigned>(it.area);  // a band's coordinates stay below 2^32
     const float2 ends = p.group[p.goff[it.b] + blockIdx.y * it.area + it.pixel];
     float lamT = ends.x;
     for (int s = it.s1 - 1; s >= it.s0; --s) {
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
         float T = ends.y * p.front[p.soff[it.b] + s * it.area + it.pixel];
         float xs[kGradSeg], Ts[kGradSeg];
 #pragma unroll
-        for (int j = 0; j < kGradSeg; ++j) xs[j] = __ldcs(x + min(j, left) * it.area);
+        for (int j = 0; j < kGradSeg; ++j) xs[j] = __ldcs(x + static_cast<unsigned>(min(j, left)) * area);
 #pragma unroll
         for (int j = 0; j < kGradSeg; ++j) {
             float w;
@@ -417,69 +424,99 @@ __global__ void __launch_bounds__(128, 5) grad_samples_kernel(const __grid_const
             const float g4[4] = {it.g.x * ta, it.g.y * ta, it.g.z * ta, Ts[j] * (gc - lamT)};
             lamT = lamT * (1.0f - a) + a * gc;
             // table: rgba = (1-w) T[i] + w T[i+1]
-            if (ti != cur_ti) next_interval(ti);
-            const float w0 = 1.0f - w;
+            const int ie = (ti + 1) & ~1, io = ti | 1;
+            if (ie != cur_e) {
+                leave(copy + cur_e, cur_e >= 0, tab_e);
+                cur_e = ie;
+            }
+            if (io != cur_o) {
+                leave(copy + cur_o, cur_o >= 0, tab_o);
+                cur_o = io;
+            }
+            const float w0 = 1.0f - w, we = ti & 1 ? w : w0, wo = ti & 1 ? w0 : w;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                at0[c] = fmaf(w0, g4[c], at0[c]);
-                at1[c] = fmaf(w, g4[c], at1[c]);
+                tab_e[c] = fmaf(we, g4[c], tab_e[c]);
+                tab_o[c] = fmaf(wo, g4[c], tab_o[c]);
             }
             // scalar: ds = (g . (T[i+1] - T[i])) dx/ds where the table coordinate is not clamped
             if (voxels && j <= left && xj > 0.0f && xj < xmax) {
                 const float ds = (g4[0] * de.x + g4[1] * de.y + g4[2] * de.z + g4[3] * de.w) * m.tf_scale;
                 GradCell q;
                 grad_cell(it.run, h0 + static_cast<float>(j), q);
-                if (q.bx != cur_x || q.by != cur_y || q.bz != cur_z) next_cell(q);
+                next_cell(q);
                 const float ux = 1.0f - q.wx, uy = 1.0f - q.wy, uz = 1.0f - q.wz;
-                const float dz0 = ds * uz, dz1 = ds * q.wz;
-                lower[0] = fmaf(dz0, ux * uy, lower[0]);
-                lower[1] = fmaf(dz0, q.wx * uy, lower[1]);
-                lower[2] = fmaf(dz0, ux * q.wy, lower[2]);
-                lower[3] = fmaf(dz0, q.wx * q.wy, lower[3]);
-                upper[0] = fmaf(dz1, ux * uy, upper[0]);
-                upper[1] = fmaf(dz1, q.wx * uy, upper[1]);
-                upper[2] = fmaf(dz1, ux * q.wy, upper[2]);
-                upper[3] = fmaf(dz1, q.wx * q.wy, upper[3]);
+                const bool odd = q.bz & 1u;
+                const float de_ = ds * (odd ? q.wz : uz), do_ = ds * (odd ? uz : q.wz);
+                pl_e[0] = fmaf(de_, ux * uy, pl_e[0]);
+                pl_e[1] = fmaf(de_, q.wx * uy, pl_e[1]);
+                pl_e[2] = fmaf(de_, ux * q.wy, pl_e[2]);
+                pl_e[3] = fmaf(de_, q.wx * q.wy, pl_e[3]);
+                pl_o[0] = fmaf(do_, ux * uy, pl_o[0]);
+                pl_o[1] = fmaf(do_, q.wx * uy, pl_o[1]);
+                pl_o[2] = fmaf(do_, ux * q.wy, pl_o[2]);
+                pl_o[3] = fmaf(do_, q.wx * q.wy, pl_o[3]);
             }
         }
     }
-    if (voxels) next_cell(GradCell{});
-    next_interval(-4);
+    if constexpr (QUADS) {
+        if (quad_e != ~0u) red_v4(gquads + quad_e, pl_e);
+        if (quad_o != ~0u) red_v4(gquads + quad_o, pl_o);
+    } else {
+        if (cur_x != 0) leave_cell();
+    }
+    if (cur_e >= 0) red_v4(copy + cur_e, tab_e);
+    if (cur_o >= 0) red_v4(copy + cur_o, tab_o);
 }
 
 // Step 4 (QUADS): every haloed voxel of every brick sums its share of the four
 // quads that hold it and adds it to the volume's voxel (halo copies alias their
-// neighbours' voxels). A warp takes one x row, 32 voxels at a time: two 16-byte
-// loads per voxel, the left neighbour's halves from the lane below. 0.08 ms for
-// 256^3 (0.28 GB of quads, 3.5 TB/s).
+// neighbours' voxels). A warp takes 31 voxels along x (lane 0 has the quad on their
+// left) and kGradVoxelRows rows: a quad is loaded once, the row below's half stays in
+// registers and the left neighbour's comes from the lane below, and the quads' index
+// is stepped. Bound by HBM:
+// 0.069 ms for 256^3 (0.28 GB of quads, 0.35 GB read with the voxels, 73% of the peak
+// DRAM rate); one row per warp, both quads of a voxel loaded and indexed anew, took
+// 0.080 ms.
 __global__ void __launch_bounds__(256) grad_voxels_kernel(const __grid_constant__ GradVoxelParams p)
 {
     int lo = 0, hi = p.nb - 1;
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (row >= p.n_rows) return;
+    const int task = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (task >= p.n_tasks) return;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (p.b[mid].row_begin <= row) lo = mid;
+        if (p.b[mid].task_begin <= task) lo = mid;
         else hi = mid - 1;
     }
     const GradVoxelBrick &B = p.b[lo];
-    const int local = row - B.row_begin;
-    const int lz = local / B.s[1], ly = local - lz * B.s[1];
+    const int local = task - B.task_begin;
+    const int nx = grad_voxel_chunks(B.s[0]), ny = grad_voxel_row_sets(B.s[1]);
+    const int yz = local / nx, cx = local - yz * nx, lz = yz / ny, y0 = (yz - lz * ny) * kGradVoxelRows;
+    const int lx = cx * 31 - 1 + lane;
     const int qx = B.s[0] - 1, qy = B.s[1] - 1, nbx = B.s[0] / 2, nby = B.s[1] / 2;
-    const float4 *quads = p.quads + B.base;
-    const int gy = min(max(B.lo[1] + ly - 1, 0), p.N[1] - 1), gz = min(max(B.lo[2] + lz - 1, 0), p.N[2] - 1);
-    float *out = p.grad_vol + (static_cast<long long>(gz) * p.N[1] + gy) * p.N[0];
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float left = 0.0f;  // from the last lane of the previous 32 quads
-    for (int x0 = 0; x0 < B.s[0]; x0 += 32) {
-        const int lx = x0 + lane;
-        const float4 a = lx < qx && ly < qy ? __ldcs(quads + quad_index(lx, ly, lz, nbx, nby)) : zero;
-        const float4 b = lx < qx && ly > 0 ? __ldcs(quads + quad_index(lx, ly - 1, lz, nbx, nby)) : zero;
-        const float own = a.x + b.z, next = a.y + b.w;
-        const float below = __shfl_up_sync(0xffffffffu, next, 1);
-        const float v = own + (lane == 0 ? left : below);
-        left = __shfl_sync(0xffffffffu, next, 31);
-        if (lx < B.s[0] && v != 0.0f) atomicAdd(out + min(max(B.lo[0] + lx - 1, 0), p.N[0] - 1), v);
+    const bool quad = lx >= 0 && lx < qx, voxel = lane > 0 && lx < B.s[0];
+    const float4 *at = p.quads + B.base + quad_index(quad ? lx : 0, y0, lz, nbx, nby);  // row y0 is even
+    const int gx = min(max(B.lo[0] + lx - 1, 0), p.N[0] - 1);
+    const int gz = min(max(B.lo[2] + lz - 1, 0), p.N[2] - 1);
+    float *out = p.grad_vol + static_cast<long long>(gz) * p.N[1] * p.N[0] + gx;
+    const long long down = 8LL * nbx;  // two rows on
+    float bz = 0.0f, bw = 0.0f;        // the row below's quad
+    if (quad && y0 > 0) {
+        const float4 b = __ldg(at + 2 - down);
+        bz = b.z;
+        bw = b.w;
+    }
+    const int y1 = min(y0 + kGradVoxelRows, B.s[1]);
+#pragma unroll 4
+    for (int ly = y0; ly < y1; ++ly) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (quad && ly < qy) a = __ldg(at + ((ly - y0) >> 1) * down + 2 * (ly & 1));
+        const float own = a.x + bz, next = a.y + bw;
+        const float v = own + __shfl_up_sync(0xffffffffu, next, 1);
+        bz = a.z;
+        bw = a.w;
+        const int gy = min(max(B.lo[1] + ly - 1, 0), p.N[1] - 1);
+        if (voxel && v != 0.0f) atomicAdd(out + static_cast<long long>(gy) * p.N[0], v);
     }
 }
 
@@ -559,8 +596,8 @@ cudaError_t launch_grad_samples(const GradParams &p, int groups, cudaStream_t s)
 
 cudaError_t launch_grad_voxels(const GradVoxelParams &p, cudaStream_t s)
 {
-    if (p.n_rows <= 0) return cudaSuccess;
-    grad_voxels_kernel<<<(p.n_rows + 7) / 8, 256, 0, s>>>(p);
+    if (p.n_tasks <= 0) return cudaSuccess;
+    grad_voxels_kernel<<<(p.n_tasks + 7) / 8, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
 

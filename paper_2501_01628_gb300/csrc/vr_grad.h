@@ -22,10 +22,10 @@ constexpr int kGradLaneCopies = 8;
 // Voxel gradients go through quads (at most two 16-byte reductions per cell, then
 // one pass over the volume's quads) when the view's samples, bounded by rect areas
 // times longest runs, are over this many times the quads, else straight into the
-// voxels (eight reductions per cell). One view, 8 bricks, us per training step quads
-// / direct: 256^3 at 256^2 (ratio 1.6) 1362 / 1287, at 384^2 (3.6 to 4.4) 1500 / 1541;
-// 128^3 at 256^2 (6.4) 1025 / 1099; 256^3, four views at 512^2 (5.8 to 7.4) 5320 / 6010.
-constexpr long long kGradQuadsRatio = 4;
+// voxels (eight reductions per cell). One backward of 8 bricks, us, quads / direct:
+// 256^3 at 256^2 (ratio 1.6) 416 / 351, at 384^2 (3.6 to 4.4) 527 / 557, at 512^2 (5.8
+// to 7.4) 692 / 865; 128^3 at 256^2 (6.4) 156 / 186; 64^3 at 256^2 118 / 155.
+constexpr long long kGradQuadsRatio = 3;
 constexpr long long kGradBandBytes = 1LL << 30;  // per-sample workspace of one band of image rows
 
 struct GradParams {
@@ -48,19 +48,23 @@ struct GradParams {
     int *error;                   // device error word: bit 0 = a run exceeded kGradMaxRun
 };
 
-// Voxel gradients gathered from the quads (grad_voxels_kernel).
+// Voxel gradients gathered from the quads (grad_voxels_kernel): a warp's task is a
+// chunk of 31 voxels along x in a set of rows of one plane.
+constexpr int kGradVoxelRows = 16;  // even: a set starts at the lower row of the quads' blocks
+__host__ __device__ inline int grad_voxel_chunks(int sx) { return (sx + 30) / 31; }
+__host__ __device__ inline int grad_voxel_row_sets(int sy) { return (sy + kGradVoxelRows - 1) / kGradVoxelRows; }
 struct GradVoxelBrick {
     long long base;   // quad offset of the brick's storage
     int lo[3];        // voxel box origin
     int s[3];         // haloed extents
-    int row_begin;    // first of the brick's s[1] x s[2] rows
+    int task_begin;   // first of the brick's s[2] x row sets x chunks
 };
 struct GradVoxelParams {
     const float4 *quads;
     float *grad_vol;
     int N[3];
     int nb;
-    int n_rows;
+    int n_tasks;
     GradVoxelBrick b[kMaxBricks];
 };
 

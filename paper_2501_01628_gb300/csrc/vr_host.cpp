@@ -1306,7 +1306,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         vp.quads = gp.grad_quads;
         vp.grad_vol = grad_density_dev;
         vp.nb = nb;
-        long long rows = 0;
+        long long tasks = 0;
         for (int a = 0; a < 3; ++a) vp.N[a] = vol->dims[a];
         for (int b = 0; b < nb; ++b) {
             const int *bx = &vol->boxes[6 * b];
@@ -1316,10 +1316,11 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
                 V.lo[a] = bx[a];
                 V.s[a] = bx[3 + a] - bx[a] + 2;
             }
-            V.row_begin = static_cast<int>(rows);
-            if (fr.rects[4 * b + 2] > 0) rows += static_cast<long long>(V.s[1]) * V.s[2];  // seen bricks only
+            V.task_begin = static_cast<int>(tasks);
+            if (fr.rects[4 * b + 2] > 0)  // seen bricks only
+                tasks += static_cast<long long>(V.s[2]) * grad_voxel_row_sets(V.s[1]) * grad_voxel_chunks(V.s[0]);
         }
-        vp.n_rows = static_cast<int>(rows);
+        vp.n_tasks = static_cast<int>(tasks);
         VR_LAUNCH(ctx, launch_grad_voxels(vp, s));
     }
     VR_LAUNCH(ctx, launch_grad_table(gp.tf_copies, ctx->ntf, grad_tf_dev, s));

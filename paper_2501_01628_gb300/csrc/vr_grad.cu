@@ -115,10 +115,7 @@ __device__ __forceinline__ float grad_value(const MarchParams &m, const typename
         a0 = Quad<S>::load(vox + c);
         a1 = Quad<S>::load(vox + c1);
     }
-    const float c00 = fmaf(q.wx, a0.y - a0.x, a0.x), c10 = fmaf(q.wx, a0.w - a0.z, a0.z);
-    const float c01 = fmaf(q.wx, a1.y - a1.x, a1.x), c11 = fmaf(q.wx, a1.w - a1.z, a1.z);
-    const float c0_ = fmaf(q.wy, c10 - c00, c00), c1_ = fmaf(q.wy, c11 - c01, c01);
-    return fmaf(fmaf(q.wz, c1_ - c0_, c0_), m.tf_scale, m.tf_bias);
+    return fmaf(dev::trilinear<S>(a0, a1, q.wx, q.wy, q.wz), m.tf_scale, m.tf_bias);
 }
 
 // The table interval of coordinate x and the weight of its upper entry.

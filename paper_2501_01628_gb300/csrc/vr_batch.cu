@@ -232,7 +232,8 @@ cudaError_t launch_batch(const BatchParams &p, int kind, int blocks, cudaStream_
     }
 }
 
-// What fits of every variant: a batch keeps its plan when the correction changes.
+// What fits of every variant, so that a choice of blocks per SM (a saved one too)
+// does not depend on the opacity correction.
 template <typename S>
 int batch_fits()
 {

@@ -419,14 +419,18 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
  * inside that box (1e-3 voxel tolerance); each brick's elements must fill its box
  * without gaps or overlaps (volumes checked to 1e-4) and share faces only
  * pairwise. A violation, a degenerate element or an empty brick gives
- * VR_ERR_ARG. The per-brick BVHs and face adjacency are built on the host.
+ * VR_ERR_ARG. Elements need not share all faces that touch: vertices may be
+ * doubled, hang on a neighbour's edge or face, or belong to one element each; rays
+ * find the element behind such a face through the BVH, which takes longer. The
+ * per-brick BVHs, start grids and face adjacency are built on the host.
  *
  * Sampling (reading; the paper gives none): a lattice sample keeps the owner of
  * the voxel path (its cell's brick) and takes the linear interpolant
  * sum_i lambda_i s_i of the owner's element containing it; rendering,
  * classification, early termination, opacity correction and compositing are
  * those of vr_render_frame (sort-last mode only). Device memory: 80 bytes per
- * element (record + neighbours) plus 32 bytes per BVH node. */
+ * element (record + neighbours), 32 bytes per BVH node and 4 bytes per cell of the
+ * start grids (about one for two elements). */
 vr_status vr_mesh_create(vr_ctx ctx, const int dims[3], const vr_partition *part, const float *verts,
                          long long n_verts, const float *values, const int *tets, long long n_tets,
                          vr_mesh *out);
@@ -435,8 +439,9 @@ vr_status vr_mesh_release(vr_mesh mesh);
  * bytes of the mesh (may be NULL). */
 vr_status vr_mesh_info(vr_mesh mesh, int *n_bricks, long long *elements_per_brick, long long *device_bytes);
 /* One frame of the mesh with the context's camera, transfer function and
- * parameters: per-brick partials (BVH point location of each ray's first owned
- * sample, then a walk through face neighbours), then the composite, into
+ * parameters: per-brick partials (each ray's first owned sample is located from
+ * the brick's start grid by a walk through face neighbours, or by its BVH where that
+ * walk does not end; then a walk along the ray), then the composite, into
  * out_rgba (H x W x 4 float32; device if out_on_device, else host). Asynchronous
  * on `stream` like vr_render_frame. VR_ERR_STATE in ray-state cycling mode. */
 vr_status vr_render_mesh_frame(vr_ctx ctx, vr_mesh mesh, float *out_rgba, int out_on_device, void *stream);

@@ -21,6 +21,13 @@
 //          walk or element steps do not end)
 //   0.404  two samples per iteration, warp-converged, the BVH outside the loop (inside,
 //          its registers spill in the loop: 0.551)
+//   0.407  a walk ends only in an element that holds the sample (without that test, in
+//          any element whose faces towards the sample have no neighbour: wrong values
+//          where vertices are doubled, hang or are not merged inside a brick). Such
+//          meshes pay for the BVH, ms with all rays located in it / now: a hundredth of
+//          the elements cut in two but not their neighbours 1.18 / 0.92, a fifth
+//          5.98 / 4.08, a vertex set per element 9.77 / 9.82 (10.83 with 128-bit record loads
+//          in the BVH's leaves, which spill 12 bytes less and leave the rest 0.3% faster)
 // Waiting until 4 to 24 lanes can step together: 0.452 to 0.461; lanes left to
 // diverge: 0.596; 6, 7, 9 blocks per SM: 0.480, 0.500, 0.717 (spills).
 #include "vr_device.cuh"
@@ -35,7 +42,9 @@ using dev::ldg_v8;
 // Smallest barycentric coordinate of q in the element (record at rec).
 __device__ __forceinline__ float min_bary(const float4 *rec, float qx, float qy, float qz)
 {
-    const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2), r3 = __ldg(rec + 3);
+    float4 r0, r1, r2, r3;
+    ldg_v8(rec, r0, r1);
+    ldg_v8(rec + 2, r2, r3);
     const float dx = qx - r0.x, dy = qy - r0.y, dz = qz - r0.z;
     const float l1 = fmaf(r1.x, dx, fmaf(r1.y, dy, fmaf(r1.z, dz, 0.25f)));
     const float l2 = fmaf(r2.x, dx, fmaf(r2.y, dy, fmaf(r2.z, dz, 0.25f)));
@@ -185,9 +194,9 @@ __global__ void __launch_bounds__(128, 8) march_mesh_kernel(const __grid_constan
                 t_exit = t + __fdividef(num, den);
                 if (walk > 0) {  // on through the face the sample lies furthest behind, if any
                     float low = -kMeshInside;
-                    int on = -1;
+                    int on = -2;  // none; -1: a face without a neighbour
                     auto behind = [&](float lam, int other) {
-                        if (other >= 0 && lam < low) {
+                        if (lam < low) {
                             low = lam;
                             on = other;
                         }
@@ -196,12 +205,15 @@ __global__ void __launch_bounds__(128, 8) march_mesh_kernel(const __grid_constan
                     behind(l1, nb.y);
                     behind(l2, nb.z);
                     behind(l3, nb.w);
-                    if (on >= 0) {
-                        nx = on;
-                        t_exit = -3.0e38f;
-                    } else {
+                    if (on == -2) {
                         walk = 0;
                         located = true;
+                    } else {
+                        // this element does not hold the sample; without a neighbour to
+                        // go to, the walk ends in the BVH
+                        nx = on < 0 ? e : on;
+                        if (on < 0) walk = 1;
+                        t_exit = -3.0e38f;
                     }
                 }
                 // a located element takes its first sample whatever the rounding says
@@ -252,8 +264,8 @@ __global__ void __launch_bounds__(128, 8) march_mesh_kernel(const __grid_constan
         }
         if (!__any_sync(0xffffffffu, lost)) break;
         if (lost) {
-            // too many steps without a sample (rounding near edges and vertices) or of
-            // a walk: a point location
+            // too many steps without a sample (rounding near edges and vertices) or of a
+            // walk, or a walk that came to a face without a neighbour: a point location
             nx = locate(P.nodes + P.node_base[bi], rec, fmaf(t, ray.dv[0], ray.ov[0]), fmaf(t, ray.dv[1], ray.ov[1]),
                         fmaf(t, ray.dv[2], ray.ov[2]));
             if (nx < 0) {

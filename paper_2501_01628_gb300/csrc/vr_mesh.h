@@ -6,9 +6,10 @@
 // (Sec. 5); elements here are tetrahedra, each held by one brick. Within an
 // element the value is linear, so along a ray it is linear in t, and a ray
 // leaves the element through the face whose barycentric coordinate reaches 0
-// first. A ray's run inside a brick therefore starts with one point location
-// (a per-brick BVH, the acceleration structure of Sec. 2.1) and then walks
-// face neighbours.
+// first. A ray's run inside a brick therefore starts with one point location (the
+// brick's start grid and a walk through face neighbours or, where that walk does
+// not end, the brick's BVH, the acceleration structure of Sec. 2.1) and then
+// walks face neighbours.
 #pragma once
 
 #include "vr_internal.h"
@@ -42,9 +43,11 @@ constexpr int kMeshStallSteps = 32;    // element steps without a sample before 
 
 // Start grid of a brick: n[0] x n[1] x n[2] equal cells of its box, each with an
 // element near the cell's centre (brick-local), from which a walk through face
-// neighbours reaches a sample in the cell in a step or two -- the bricks are
-// convex and filled, so the walk towards the sample always has a neighbour.
-// About kMeshGridElems elements per cell.
+// neighbours reaches a sample in the cell in a step or two. Bricks are convex and
+// filled, so where all faces inside a brick are shared the walk always has a
+// neighbour to go to. Vertices doubled on an interior surface, hanging nodes or
+// unmerged vertices leave faces inside that no second element shares: a walk that
+// comes to one ends in the BVH. About kMeshGridElems elements per cell.
 struct MeshGrid {
     long long base;   // first cell in MeshParams::start
     int n[3];
@@ -57,7 +60,7 @@ constexpr float kMeshInside = 1.0e-6f; // barycentric slack of a sample on a fac
 struct MeshParams {
     MarchParams m;                    // camera, lattice, transfer function, tiles, bricks
     const float4 *rec;                // kMeshRec float4 per element
-    const int4 *nbr;                  // brick-local neighbour across face i, -1 on the brick's boundary
+    const int4 *nbr;                  // brick-local neighbour across face i, -1 if no element of the brick shares it
     const MeshNode *nodes;
     const int *start;                 // start grids
     MeshGrid grid[kMaxBricks];

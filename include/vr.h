@@ -396,7 +396,17 @@ vr_status vr_volume_update_async(vr_volume vol, const float *src, int src_on_dev
  * never from division. Requires early termination off (VR_ERR_ARG otherwise).
  * Runs of more than 4096 owned samples in one brick are skipped and reported as
  * VR_ERR_BOUNDS by vr_sync. Float atomics: results vary in the last bits
- * between runs. */
+ * between runs.
+ * Device memory, kept for the next call and given back when an allocation of the
+ * context finds no room: a workspace of about 4.7 bytes per sample of the view (counted
+ * as footprint areas times longest runs; at most about 1.2 GiB, larger views go in
+ * bands of rows) until vr_destroy, and, where grad_density_dev is given and the view
+ * has many samples against the volume's cells, 16 bytes per cell of the haloed bricks
+ * (0.28 GB for 256^3, 17 GB for 1024^3; vr_volume_info's bytes do not count them) until
+ * vr_volume_release. Where the first cannot be had the bands are smaller, where
+ * the second cannot be had the voxels' sums are made without it: slower, the same
+ * result. A graph captured around the call holds the memory's addresses: replay it
+ * only while they are kept. */
 vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_dev, float *grad_tf_dev,
                              float *grad_density_dev, void *stream);
 

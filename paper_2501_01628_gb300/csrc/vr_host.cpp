@@ -37,7 +37,7 @@ bool fault_now(int kind)
     return true;
 }
 
-cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes)
+cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes, bool give_backward)
 {
     cudaError_t e = dev_malloc(p, bytes);
     if (e == cudaErrorMemoryAllocation && ctx->spare) {
@@ -45,6 +45,19 @@ cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes)
         cudaFree(ctx->spare);
         ctx->spare = nullptr;
         ctx->spare_px = 0;
+        e = dev_malloc(p, bytes);
+    }
+    if (e == cudaErrorMemoryAllocation && give_backward && (ctx->d_grad || !ctx->quad_vols.empty())) {
+        cudaGetLastError();
+        cudaDeviceSynchronize();  // a backward may still be using it
+        cudaFree(ctx->d_grad);
+        ctx->d_grad = nullptr;
+        ctx->grad_cap = 0;
+        for (vr_volume v : ctx->quad_vols) {
+            cudaFree(v->d_gquads);
+            v->d_gquads = nullptr;
+        }
+        ctx->quad_vols.clear();
         e = dev_malloc(p, bytes);
     }
     return e;
@@ -1285,9 +1298,17 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     gp.grad_quads = nullptr;
     const long long quads = vol->quad_bytes / static_cast<long long>(quad_size(vol->dtype, vol->octets));
     if (grad_density_dev && view_segs * kGradSeg > kGradQuadsRatio * quads) {
-        if (!vol->d_gquads && vr::host::dev_malloc(ctx, &vol->d_gquads, quads * sizeof(float4)) != cudaSuccess)
-            cudaGetLastError();  // no room: reductions straight into the voxels
-        gp.grad_quads = vol->d_gquads;
+        const size_t bytes = static_cast<size_t>(quads) * sizeof(float4);
+        if (!vol->d_gquads) {
+            void *got = nullptr;
+            if (vr::host::dev_malloc_bytes(ctx, &got, bytes, false) == cudaSuccess) {
+                vol->d_gquads = static_cast<float4 *>(got);
+                ctx->quad_vols.push_back(vol);
+            } else {
+                cudaGetLastError();
+            }
+        }
+        gp.grad_quads = vol->d_gquads;  // null: reductions straight into the voxels
     }
     for (int a = 0; a < 3; ++a) gp.N[a] = vol->dims[a];
     gp.error = ctx->d_error;
@@ -1335,6 +1356,8 @@ vr_status vr_volume_release(vr_volume vol)
     cudaFree(vol->d_staging);
     cudaFree(vol->d_scalar);
     cudaFree(vol->d_gquads);
+    std::vector<vr_volume> &quads = vol->ctx->quad_vols;
+    quads.erase(std::remove(quads.begin(), quads.end(), vol), quads.end());
     vol->ctx->live_objects--;
     delete vol;
     return VR_OK;

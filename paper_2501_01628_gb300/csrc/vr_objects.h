@@ -27,8 +27,9 @@ cudaError_t dev_malloc(T **p, size_t bytes)
     return cudaMalloc(reinterpret_cast<void **>(p), bytes);
 }
 
-// The same, giving the context's spare frame memory back if there is no room.
-cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes);
+// The same, giving back what the context keeps for later calls if there is no room:
+// its spare frame memory, then (unless the call is using it) the backward's.
+cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes, bool give_backward = true);
 template <typename T>
 cudaError_t dev_malloc(vr_ctx ctx, T **p, size_t bytes)
 {
@@ -109,6 +110,7 @@ struct vr_ctx_s {
     bool count_samples = false;
     char *d_grad = nullptr;        // backward workspace: table copies, segments, segment counts
     size_t grad_cap = 0;           // bytes
+    std::vector<vr_volume> quad_vols;  // volumes that hold quads of voxel gradients
     vr_frame_s frame;              // context-owned frame for vr_render_frame
     // Memory of the last released frame of vr_render_partials, for the next one
     // (partials, composite and release of a 1023 x 767 frame of 27 bricks: 0.480 ms

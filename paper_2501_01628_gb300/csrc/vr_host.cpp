@@ -63,6 +63,26 @@ cudaError_t dev_malloc_bytes(vr_ctx ctx, void **p, size_t bytes, bool give_backw
     return e;
 }
 
+size_t device_room()
+{
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) != cudaSuccess) cudaGetLastError();
+    return room;
+}
+
+void refuse(Refused &r, size_t bytes)
+{
+    r.bytes = bytes;
+    r.room = device_room();
+}
+
+// Whether `bytes` are worth asking for, `held` bytes being given up for them: not
+// while there is hardly more room than when as much was refused.
+bool worth_asking(const Refused &r, size_t bytes, size_t held)
+{
+    return r.bytes == 0 || bytes < r.bytes || device_room() + held >= std::max(bytes, r.room + bytes / 8);
+}
+
 size_t elem_size(vr_dtype t) { return t == VR_F32 ? 4 : 2; }
 // bytes of one xy-quad (four voxels) in device storage
 // bytes of one storage element: an xy-quad (four voxels), or an octet (both
@@ -1255,7 +1275,8 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     };
     // workspace: table copies, groups, samples, segments, counts (each part a
     // multiple of 16 bytes from the start); bands of rows where a view's samples do
-    // not fit its bound or it cannot be had
+    // not fit its bound or it cannot be had. A size once refused is not asked for again
+    // while the device has no more room: the smaller one at hand stays
     auto part = [](long long n, size_t size) { return (static_cast<size_t>(n) * size + 15) & ~static_cast<size_t>(15); };
     const size_t copies_bytes = part(static_cast<long long>(kGradCopies) * (ctx->ntf + 1), sizeof(float4));
     size_t group_bytes, x_bytes, front_bytes;
@@ -1276,6 +1297,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         front_bytes = part(most.segs, sizeof(float));
         const size_t need = copies_bytes + group_bytes + x_bytes + front_bytes + part(most.px, sizeof(unsigned short));
         if (need <= ctx->grad_cap) break;
+        if (band_h > 1 && !vr::host::worth_asking(ctx->grad_refused, need, ctx->grad_cap)) continue;
         cudaFree(ctx->d_grad);
         ctx->d_grad = nullptr;
         ctx->grad_cap = 0;
@@ -1286,6 +1308,7 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
         }
         if (e != cudaErrorMemoryAllocation || band_h <= 1) return cuda_fail(ctx, e, "backward workspace");
         cudaGetLastError();
+        vr::host::refuse(ctx->grad_refused, need);
     }
     char *at = ctx->d_grad;
     gp.tf_copies = reinterpret_cast<float *>(at);
@@ -1299,13 +1322,14 @@ vr_status vr_render_backward(vr_ctx ctx, vr_volume vol, const float *grad_rgba_d
     const long long quads = vol->quad_bytes / static_cast<long long>(quad_size(vol->dtype, vol->octets));
     if (grad_density_dev && view_segs * kGradSeg > kGradQuadsRatio * quads) {
         const size_t bytes = static_cast<size_t>(quads) * sizeof(float4);
-        if (!vol->d_gquads) {
+        if (!vol->d_gquads && vr::host::worth_asking(vol->gquads_refused, bytes, 0)) {
             void *got = nullptr;
             if (vr::host::dev_malloc_bytes(ctx, &got, bytes, false) == cudaSuccess) {
                 vol->d_gquads = static_cast<float4 *>(got);
                 ctx->quad_vols.push_back(vol);
             } else {
                 cudaGetLastError();
+                vr::host::refuse(vol->gquads_refused, bytes);
             }
         }
         gp.grad_quads = vol->d_gquads;  // null: reductions straight into the voxels

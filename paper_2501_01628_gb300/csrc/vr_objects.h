@@ -36,6 +36,14 @@ cudaError_t dev_malloc(vr_ctx ctx, T **p, size_t bytes)
     return dev_malloc_bytes(ctx, reinterpret_cast<void **>(p), bytes);
 }
 
+// A refused request for memory that a call can do with less of (or without): what was
+// asked for and what the device had free. Asked for again at every call, it would cost
+// a failing allocation each time.
+struct Refused {
+    size_t bytes = 0;  // the smallest such request (0: none)
+    size_t room = 0;
+};
+
 // Named NVTX range around a public call (visible in timeline profilers; a no-op
 // unless a tool is attached).
 struct TraceRange {
@@ -110,6 +118,7 @@ struct vr_ctx_s {
     bool count_samples = false;
     char *d_grad = nullptr;        // backward workspace: table copies, segments, segment counts
     size_t grad_cap = 0;           // bytes
+    vr::host::Refused grad_refused;
     std::vector<vr_volume> quad_vols;  // volumes that hold quads of voxel gradients
     vr_frame_s frame;              // context-owned frame for vr_render_frame
     // Memory of the last released frame of vr_render_partials, for the next one
@@ -170,6 +179,7 @@ struct vr_volume_s {
     long long quad_bytes = 0;      // of them the bricks' quads (or octets)
     float *d_staging = nullptr;    // float32 source for asynchronous re-packs from host memory
     float4 *d_gquads = nullptr;    // quads of voxel gradients (vr_render_backward), laid out as d_data
+    vr::host::Refused gquads_refused;
     // scalar copy of the bricks for the staged march (float32 volumes created
     // while the context's staging was on): per brick, haloed voxels with rows
     // padded to sxp elements, starting at element sbase

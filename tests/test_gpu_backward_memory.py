@@ -1,5 +1,7 @@
-"""An allocation that finds no room while vr_render_backward's memory is kept, with the
-failure injected on the host. Every gradient against the oracle's FP64 adjoint."""
+"""vr_render_backward's memory where there is no room: a workspace or quads that
+cannot be had, and what is not asked for again after that; and another allocation
+that finds no room while the backward's memory is kept. The failures are injected
+on the host. Every gradient against the oracle's FP64 adjoint."""
 import numpy as np
 import pytest
 
@@ -25,7 +27,8 @@ def vr():
 
 @pytest.fixture()
 def scene(vr):
-    """backward() checks the gradients of a context's volume."""
+    """backward() checks the gradients of a context's volume; pending() tells whether an
+    injected fault is still to come (and clears it)."""
     import torch
     rng = np.random.default_rng(12)
     vol = synth.blob_volume(40, synth.draw_blobs(rng, 5))[:SHAPE[0], :SHAPE[1], :SHAPE[2]].copy()
@@ -36,7 +39,7 @@ def scene(vr):
     G = rng.standard_normal((SIZE[1], SIZE[0], 4)).astype(np.float32)
     boxes = vr.vr_partition_boxes(SHAPE[::-1], PART)
     want = oracle.render_grad(vol, boxes, tf, 0.0, 1.0, cam, G, 0.5)
-    ctx = vr.vr_create(0)
+    ctx, bare = vr.vr_create(0), vr.vr_create(0)
     v = vr.vr_volume_create(ctx, vol, "f32", PART)
     vr.vr_set_transfer_function(ctx, tf, 0.0, 1.0)
     vr.vr_set_camera(ctx, cam)
@@ -50,15 +53,36 @@ def scene(vr):
         for got, ref in zip((gtf, gvol), want):
             assert np.linalg.norm(got.cpu().numpy() - ref) <= REL * np.linalg.norm(ref)
 
-    yield ctx, v, cam, backward
+    def pending():
+        try:
+            vr.vr_volume_release(vr.vr_volume_create(bare, vol, "f32", PART))  # nothing to give back there
+        except vr.VrError as e:
+            assert e.status == vr.VR_ERR_OOM
+            return True
+        return False
+
+    yield ctx, v, cam, backward, pending
     vr.vr_debug_inject_fault(vr.VR_FAULT_NONE, 0)
     vr.vr_volume_release(v)
     vr.vr_destroy(ctx)
+    vr.vr_destroy(bare)
+
+
+@pytest.mark.parametrize("refused", [0, 1])  # the workspace; the quads
+def test_refused_memory_is_done_without_and_not_asked_for_again(vr, scene, refused):
+    _, _, _, backward, pending = scene
+    vr.vr_debug_inject_fault(vr.VR_FAULT_ALLOC, refused)
+    backward()
+    assert not pending()
+    vr.vr_debug_inject_fault(vr.VR_FAULT_ALLOC, 0)
+    backward()
+    assert pending()
+    backward()
 
 
 def test_kept_memory_is_given_back(vr, scene):
     import torch
-    ctx, v, cam, backward = scene
+    ctx, v, cam, backward, _ = scene
     big = synth.orbit_camera(800, 600, 40.0, elevation_deg=-15.0)
     vr.vr_set_camera(ctx, big)
     grad = torch.rand((600, 800, 4), device="cuda")

@@ -463,7 +463,12 @@ vr_status vr_render_mesh_frame(vr_ctx ctx, vr_mesh mesh, float *out_rgba, int ou
  * VR_FAULT_ALLOC) or kernel launches (kind VR_FAULT_LAUNCH) made by the library
  * in this process, the next one fails on the host without calling CUDA: the
  * call in progress returns VR_ERR_OOM or VR_ERR_CUDA with a message naming the
- * injected fault, and the context and its objects stay usable. The plan is
+ * injected fault, and the context and its objects stay usable. Two failures
+ * are made good by the library itself, as real ones are, and the call succeeds: an
+ * allocation is tried again where the context has memory to give back (of a released
+ * vr_render_partials frame, or of vr_render_backward), and vr_render_backward goes on
+ * with smaller bands or without its quads. To see a call fail, inject into a context
+ * that has released no frame and run no backward. The plan is
  * one-shot and process-wide; VR_FAULT_NONE clears it. No GPU fault is raised:
  * nothing is launched or allocated in place of the failed operation.
  * VR_ERR_ARG for an unknown kind or a negative count. */

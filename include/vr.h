@@ -35,7 +35,10 @@
  *   - Pointers named *_dev are device pointers owned by the caller; the
  *     library never frees them. Objects created by vr_*_create / vr_render_*
  *     are owned by the library until the matching release call.
- *   - A context is not thread-safe; use one context per host thread.
+ *   - A context is not thread-safe; use one context per host thread. Its table,
+ *     partial images and workspaces serve one call's work at a time: calls on
+ *     different streams must be ordered by the caller (events), except where a call
+ *     says that it waits.
  *   - Images are row-major [height][width][4] float32 RGBA, row 0 at the
  *     bottom of the view (pixel (px,py) has its centre at ((px+.5)/W, (py+.5)/H)
  *     of the image plane).

@@ -1,6 +1,6 @@
 """Differentiable rendering through libvr: a torch.autograd.Function whose
 forward is vr_render_frame and whose backward is vr_render_backward (the
-checkpointed adjoint kernels). Argument marshalling only; no pixel or gradient
+adjoint kernels). Argument marshalling only; no pixel or gradient
 arithmetic happens in Python.
 
     r = Renderer(partition=dict(kind="grid", grid=(2, 2, 2)), vmin=0.0, vmax=1.5)
@@ -19,7 +19,11 @@ from . import vr
 
 class Renderer:
     """One context plus one packed volume, re-packed when the density tensor
-    changes (data pointer or version)."""
+    changes (data pointer or version).
+
+    Renders may come from any stream: the context's table, volume and partial images
+    serve one render at a time, so a render on another stream than the last one's waits
+    (on the device) until that one is done. One host thread at a time."""
 
     def __init__(self, partition: dict, vmin: float, vmax: float, step_voxels: float = 0.5,
                  device: int | None = None, storage: str = "f32"):
@@ -32,9 +36,26 @@ class Renderer:
         self.vol = None
         self._key = None
         self._shape = None
+        self._done = None      # event behind the last render
+        self._stream = None    # its stream (None: no render, or one that is known to be done)
         vr.vr_set_render_params(self.ctx, self.step, 1.0)
 
-    def _bind(self, tf: torch.Tensor, density: torch.Tensor, cam: dict):
+    def _enter(self):
+        """The current stream, behind the last render if that was on another one. (A
+        capture starts with an idle device, and its events mean nothing outside.)"""
+        stream = torch.cuda.current_stream()
+        if self._stream is not None and stream != self._stream and not torch.cuda.is_current_stream_capturing():
+            stream.wait_event(self._done)
+        return stream
+
+    def _leave(self, stream):
+        if not torch.cuda.is_current_stream_capturing():
+            if self._done is None:
+                self._done = torch.cuda.Event()
+            self._done.record(stream)
+            self._stream = stream
+
+    def _bind(self, tf: torch.Tensor, density: torch.Tensor, cam: dict, stream):
         d = density.detach()
         if not (d.is_cuda and d.dtype == torch.float32 and d.is_contiguous()):
             raise ValueError("density must be a contiguous CUDA float32 tensor")
@@ -50,7 +71,7 @@ class Renderer:
         table = tf.detach().contiguous()
         if table.is_cuda and table.dtype == torch.float32 and table.data_ptr() % 16 == 0:
             vr.vr_set_transfer_function_async(self.ctx, table, self.vmin, self.vmax)
-            table.record_stream(torch.cuda.current_stream())
+            table.record_stream(stream)
         else:
             vr.vr_set_transfer_function(self.ctx, table, self.vmin, self.vmax)
         vr.vr_set_camera(self.ctx, cam)
@@ -76,9 +97,13 @@ class Renderer:
 class _Render(torch.autograd.Function):
     @staticmethod
     def forward(ctx, tf, density, renderer: Renderer, cam: dict):
-        renderer._bind(tf, density, cam)
-        out = torch.empty((cam["height"], cam["width"], 4), dtype=torch.float32, device=density.device)
-        vr.vr_render_frame(renderer.ctx, renderer.vol, out)
+        stream = renderer._enter()
+        try:
+            renderer._bind(tf, density, cam, stream)
+            out = torch.empty((cam["height"], cam["width"], 4), dtype=torch.float32, device=density.device)
+            vr.vr_render_frame(renderer.ctx, renderer.vol, out)
+        finally:
+            renderer._leave(stream)
         ctx.save_for_backward(tf, density)
         ctx.renderer = renderer
         ctx.cam = cam
@@ -88,9 +113,15 @@ class _Render(torch.autograd.Function):
     def backward(ctx, grad_out):
         tf, density = ctx.saved_tensors
         r = ctx.renderer
-        r._bind(tf, density, ctx.cam)
-        gtf = torch.zeros_like(tf, dtype=torch.float32)
-        gden = torch.zeros_like(density) if ctx.needs_input_grad[1] else None
-        vr.vr_render_backward(r.ctx, r.vol, grad_out.contiguous().float(), gtf, gden)
-        vr.vr_sync(r.ctx)
+        stream = r._enter()
+        try:
+            r._bind(tf, density, ctx.cam, stream)
+            gtf = torch.zeros_like(tf, dtype=torch.float32)
+            gden = torch.zeros_like(density) if ctx.needs_input_grad[1] else None
+            vr.vr_render_backward(r.ctx, r.vol, grad_out.contiguous().float(), gtf, gden)
+            vr.vr_sync(r.ctx)
+        except Exception:
+            r._leave(stream)
+            raise
+        r._stream = None
         return (gtf if ctx.needs_input_grad[0] else None), gden, None, None

@@ -398,6 +398,12 @@ cudaError_t pack_bricks(vr_volume vol, const float *dsrc, cudaStream_t s)
         }
         B.block_begin = static_cast<int>(blocks);
         B.row = 0;
+        const int width = bx[3] - bx[0];
+        B.narrow = width <= (vol->octets ? kPackNarrowOctets : kPackNarrow) && 4 * width <= vol->dims[0];
+        const int nbx = B.s[0] / 2, nby = B.s[1] / 2, step = B.narrow ? kPackStepNarrow : kPackStep;
+        B.step[0] = step % nbx;
+        B.step[1] = step / nbx % nby;
+        B.step[2] = step / nbx / nby;
         blocks += (B.quads + kPackChunk - 1) / kPackChunk;
     }
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;

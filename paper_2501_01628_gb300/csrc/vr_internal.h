@@ -226,6 +226,19 @@ struct ImagesParams {
 // from that brick's block_begin) writes the brick's storage quads
 // [j*kPackChunk, (j+1)*kPackChunk), in storage order.
 constexpr int kPackChunk = 1024;
+// A thread writes two quads in turn, or one in narrow bricks, and goes on by this many
+// 2x2x2 blocks.
+constexpr int kPackStep = 64, kPackStepNarrow = 32;
+// Bricks of at most this many voxels along x, in rows of four times as many at least. A
+// warp with two quads per thread reads twice the rows of the volume per load
+// instruction, three loads per row instead of two: a row of a narrow brick is in one or
+// two sectors, so its loads are bound by the rows, wider ones by their bytes. 512 x 512 x 128 in
+// equal bricks, us, two / one quads per thread, f32 | bf16 quads | f16 octets: 1 wide 704 /
+// 502 | 680 / 476 | 1344 / 923, 4 wide 279 / 250 | 250 / 216 | 451 / 380, 5 wide 203 / 182
+// | 183 / 160 | 345 / 293, 6 wide 192 / 193 | 154 / 165 | 274 / 239, 12 wide octets
+// 225 / 206, 16 wide 203 / 209; half of a row of 16 (165 / 170 | 117 / 134 | 185 / 201) and whole
+// rows of any width are faster with two.
+constexpr int kPackNarrow = 5, kPackNarrowOctets = 12;
 struct PackBrick {
     void *dst;             // the brick's storage
     long long quads;       // quads in the brick's storage (whole 2x2x2 blocks)
@@ -233,6 +246,8 @@ struct PackBrick {
     int s[3];              // haloed extents (the brick stores (s0-1)(s1-1)s2 quads)
     int block_begin;       // first block of this brick
     int row;               // scalar copies: padded row length in elements (multiple of 4)
+    bool narrow;           // one quad per thread (else two)
+    int step[3];           // kPackStep (narrow: kPackStepNarrow) blocks on, as blocks along x, rows, planes
 };
 struct PackParams {
     const float *src;      // x-fastest float32 volume

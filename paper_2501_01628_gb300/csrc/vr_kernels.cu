@@ -26,13 +26,14 @@ using dev::find_brick;
 //
 // Bound by memory: the volume once and the quads once (384^3: 0.23 + 0.93 GB). A
 // thread writes the two quads (i, i + 1) that share a sector: six loads for eight
-// voxels, one store. Its place in the storage is divided out once and then
-// stepped, and kPackUnroll pairs' loads are in flight together. 384^3 in 12
-// bricks: 0.190 ms, 6.0 TB/s (88% of a device copy); with one quad per thread 0.204,
-// and with two 64-bit divisions per quad, most of its instructions, 0.263.
+// voxels, one store (one quad in narrow bricks, see kPackNarrow). Its place in the
+// storage is divided out once and then stepped by the brick's PackBrick::step, and all its
+// loads are in flight together. 384^3 in 12 bricks: 0.190 ms, 6.0 TB/s (88% of
+// a device copy); with one quad per thread 0.204, and with two 64-bit divisions per
+// quad, most of its instructions, 0.263. A step that carried row by row took
+// 64 turns in a brick one block wide (2048 x 2048 x 1: 52.5 us, now 27.4).
 // ---------------------------------------------------------------------------
-constexpr int kPackThreads = 256, kPackUnroll = 2;
-static_assert(kPackChunk % (2 * kPackThreads * kPackUnroll) == 0, "whole rounds per block");
+constexpr int kPackThreads = 256;
 // two consecutive elements at an address aligned to both
 __device__ __forceinline__ void store_pair(float4 *p, const float4 &a, const float4 &b)
 {
@@ -50,6 +51,78 @@ __device__ __forceinline__ void store_pair(uint2 *p, const uint2 &a, const uint2
 {
     *reinterpret_cast<uint4 *>(p) = make_uint4(a.x, a.y, b.x, b.y);
 }
+// One block's chunk of a brick, E consecutive quads (1 or 2) per thread and round.
+template <typename T, int E>
+__device__ __forceinline__ void pack_chunk(const PackParams &p, const PackBrick &B, int chunk)
+{
+    constexpr int kRound = E * kPackThreads;         // quads per round of the block
+    constexpr int kUnroll = kPackChunk / kRound;     // rounds, their loads in flight together
+    static_assert(kRound / 8 == (E == 2 ? kPackStep : kPackStepNarrow), "2x2x2 blocks per round");
+    using Q = typename Quad<T>::type;
+    Q *dst = static_cast<Q *>(B.dst);
+    const int qx = B.s[0] - 1, qy = B.s[1] - 1, nbx = B.s[0] / 2, nby = B.s[1] / 2;
+    // a brick holds less than 2^31 quads; inverse of quad_index for the thread's first
+    const unsigned q = static_cast<unsigned>(chunk) * kPackChunk + E * threadIdx.x;
+    const unsigned q1 = static_cast<unsigned>(B.quads);
+    const unsigned bl = q >> 3, rest = bl / static_cast<unsigned>(nbx);
+    int bx = static_cast<int>(bl - rest * nbx), bz = static_cast<int>(rest / static_cast<unsigned>(nby));
+    int by = static_cast<int>(rest) - bz * nby;
+    const int ox = static_cast<int>(q & 1), oy = static_cast<int>((q >> 1) & 1), oz = static_cast<int>((q >> 2) & 1);
+    constexpr int kPlanes = Quad<T>::octet ? 2 : 1;
+    float v[kUnroll][kPlanes][2][E + 1];  // plane, row, x .. x + E
+    bool in[kUnroll], both[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+        const int lx = 2 * bx + ox, ly = 2 * by + oy, lz = 2 * bz + oz;
+        in[u] = q + u * kRound < q1 && lx < qx && ly < qy && lz < B.s[2];
+        both[u] = in[u] && E == 2 && lx + 1 < qx;
+        if (in[u]) {
+            int gx[E + 1];
+#pragma unroll
+            for (int i = 0; i <= E; ++i) gx[i] = min(max(B.lo[0] + lx - 1 + i, 0), p.N[0] - 1);
+#pragma unroll
+            for (int k = 0; k < kPlanes; ++k) {  // plane lz, and for octets plane lz + 1
+                const int gz = min(max(B.lo[2] + lz - 1 + k, 0), p.N[2] - 1);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int gy = min(max(B.lo[1] + ly - 1 + j, 0), p.N[1] - 1);
+                    const float *row = p.src + (static_cast<long long>(gz) * p.N[1] + gy) * p.N[0];
+#pragma unroll
+                    for (int i = 0; i <= E; ++i) v[u][k][j][i] = __ldg(row + gx[i]);
+                }
+            }
+        }
+        bx += B.step[0];  // the next round's 2x2x2 block
+        by += B.step[1];
+        bz += B.step[2];
+        if (bx >= nbx) {
+            bx -= nbx;
+            ++by;
+        }
+        if (by >= nby) {
+            by -= nby;
+            ++bz;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+        if (!in[u]) continue;
+        Q e[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const float (&a)[2][E + 1] = v[u][0], (&b)[2][E + 1] = v[u][kPlanes - 1];
+            if constexpr (Quad<T>::octet)
+                e[i] = Quad<T>::make8(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1], b[0][i], b[0][i + 1], b[1][i],
+                                      b[1][i + 1]);
+            else
+                e[i] = Quad<T>::make(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1]);
+        }
+        Q *d = dst + q + u * kRound;
+        if (both[u]) store_pair(d, e[0], e[E - 1]);
+        else *d = e[0];
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ PackParams p)
 {
@@ -61,69 +134,8 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constan
         else hi = mid - 1;
     }
     const PackBrick &B = p.b[lo];
-    using Q = typename Quad<T>::type;
-    Q *dst = static_cast<Q *>(B.dst);
-    const int qx = B.s[0] - 1, qy = B.s[1] - 1, nbx = B.s[0] / 2, nby = B.s[1] / 2;
-    // a brick holds less than 2^31 quads; inverse of quad_index for the pair's first
-    unsigned q = static_cast<unsigned>(blk - B.block_begin) * kPackChunk + 2 * threadIdx.x;
-    const unsigned q1 = static_cast<unsigned>(B.quads);
-    const unsigned bl = q >> 3, rest = bl / static_cast<unsigned>(nbx);
-    int bx = static_cast<int>(bl - rest * nbx), bz = static_cast<int>(rest / static_cast<unsigned>(nby));
-    int by = static_cast<int>(rest) - bz * nby;
-    const int oy = static_cast<int>((q >> 1) & 1), oz = static_cast<int>((q >> 2) & 1);
-    constexpr int kPlanes = Quad<T>::octet ? 2 : 1;
-    for (int r = 0; r < kPackChunk / (2 * kPackThreads * kPackUnroll); ++r) {
-        float v[kPackUnroll][kPlanes][2][3];  // plane, row, x .. x + 2
-        bool in[kPackUnroll], both[kPackUnroll];
-#pragma unroll
-        for (int u = 0; u < kPackUnroll; ++u) {
-            const int lx = 2 * bx, ly = 2 * by + oy, lz = 2 * bz + oz;
-            in[u] = q + 2 * u * kPackThreads < q1 && lx < qx && ly < qy && lz < B.s[2];
-            both[u] = in[u] && lx + 1 < qx;
-            if (in[u]) {
-                int gx[3];
-#pragma unroll
-                for (int i = 0; i < 3; ++i) gx[i] = min(max(B.lo[0] + lx - 1 + i, 0), p.N[0] - 1);
-#pragma unroll
-                for (int k = 0; k < kPlanes; ++k) {  // plane lz, and for octets plane lz + 1
-                    const int gz = min(max(B.lo[2] + lz - 1 + k, 0), p.N[2] - 1);
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const int gy = min(max(B.lo[1] + ly - 1 + j, 0), p.N[1] - 1);
-                        const float *row = p.src + (static_cast<long long>(gz) * p.N[1] + gy) * p.N[0];
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) v[u][k][j][i] = __ldg(row + gx[i]);
-                    }
-                }
-            }
-            bx += kPackThreads / 4;  // the next round's 2x2x2 block
-            while (bx >= nbx) {
-                bx -= nbx;
-                if (++by == nby) {
-                    by = 0;
-                    ++bz;
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kPackUnroll; ++u) {
-            if (!in[u]) continue;
-            Q e[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float (&a)[2][3] = v[u][0], (&b)[2][3] = v[u][kPlanes - 1];
-                if constexpr (Quad<T>::octet)
-                    e[i] = Quad<T>::make8(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1], b[0][i], b[0][i + 1], b[1][i],
-                                          b[1][i + 1]);
-                else
-                    e[i] = Quad<T>::make(a[0][i], a[0][i + 1], a[1][i], a[1][i + 1]);
-            }
-            Q *d = dst + q + 2 * u * kPackThreads;
-            if (both[u]) store_pair(d, e[0], e[1]);
-            else *d = e[0];
-        }
-        q += 2 * kPackThreads * kPackUnroll;
-    }
+    if (B.narrow) pack_chunk<T, 1>(p, B, blk - B.block_begin);
+    else pack_chunk<T, 2>(p, B, blk - B.block_begin);
 }
 
 // ---------------------------------------------------------------------------

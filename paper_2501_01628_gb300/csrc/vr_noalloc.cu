@@ -29,8 +29,9 @@ constexpr size_t kScratchBytes = VR_NOALLOC_SCRATCH_BYTES;
 constexpr size_t kTfBytes = 2 * 1024 * sizeof(float4);
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
-// Work item of the march: a block's 4 x 4 pixels (kGlobalLanes lanes each).
-constexpr int kGlobalTileW = 4, kGlobalTileH = 4;
+// Work item of the march: a block's pixels, LANES lanes each.
+__host__ __device__ constexpr int tile_w(int lanes) { return lanes == 1 ? 16 : lanes == 8 ? 4 : 8; }
+__host__ __device__ constexpr int tile_h(int lanes) { return kMaskThreads / lanes / tile_w(lanes); }
 
 // Device address of g_scratch on the current device. The host-side symbol is
 // not a device address; the lookup is repeated on every call (it is cheap once
@@ -46,24 +47,18 @@ cudaError_t scratch_address(void **out)
 // extents p.N). Ray setup, lattice, ownership and samples as in the
 // packed-brick march; the grid's first blocks write the composite's tile masks.
 //
-// kGlobalLanes neighbouring lanes take consecutive samples of one ray. The scratch
-// holds a few waves of work at most, often less than one, so the time is that of
-// the longest rays: with one lane per ray a sample waits for its loads, its
-// table entry and the sample before it, some 1200 cycles each. And in an x-fastest
-// volume a warp's 32 rays can lie on 32 different rows, each scalar load then
-// costs 32 wavefronts of the L1; consecutive samples of a ray share rows. The
-// transmittance runs through the lanes' samples in order (each lane repeats the
-// chain over the group's opacities); the colours are summed per lane and added
-// at the end. Bound by issue (52%) and the L1 data pipe (54%) where the image fills
-// the chip. us per call, 1 / 2 / 4 / 8 / 16 lanes per ray: 128^3, 400 x 300, six
-// bricks 244 / 130 / 83 / 76 / 82; 192^3, 400 x 320, four bricks - / - / 139 / 103 /
-// -; up to 64^3 the host's 39 us per call bound it. With one lane per ray, four
-// samples at a time took 244, keeping the cell's voxels and loading only new faces
-// 190 (divergent).
-constexpr int kGlobalLanes = 8;
-static_assert(kGlobalTileW * kGlobalTileH * kGlobalLanes == 128, "a block is one tile");
+// LANES neighbouring lanes take consecutive samples of one ray (see lanes_per_ray for
+// how many). The transmittance runs through the lanes' samples in order (each lane
+// repeats the chain over the group's opacities); the colours are summed per lane and
+// added at the end. Bound by issue (52%) and the L1 data pipe (54%) where eight lanes
+// fill the chip, by the latency of the voxels' loads else: at 9 blocks per SM (56 registers)
+// all eight are in flight, at 10 and 12 the compiler puts some behind others (384^3 along z,
+// 800 x 600, step 2, one lane: 432 / 623 / 885 us). With one lane per ray, four samples at a
+// time gained nothing, keeping the cell's voxels and loading only new faces a
+// fifth (divergent).
 static_assert(kMaskThreads == 128, "mask blocks are march blocks");
-__global__ void __launch_bounds__(128) march_global_kernel(const __grid_constant__ MarchParams p)
+template <int LANES>
+__global__ void __launch_bounds__(128, 9) march_global_kernel(const __grid_constant__ MarchParams p)
 {
     if (static_cast<int>(blockIdx.x) < p.mask_blocks) {
         dev::write_tile_mask(blockIdx.x * kMaskThreads + threadIdx.x, p.mask_tiles_x, p.mask_tiles_y, p.nb, p.order,
@@ -77,9 +72,15 @@ __global__ void __launch_bounds__(128) march_global_kernel(const __grid_constant
     const BrickLaunch &B = p.b[dev::find_brick(p, item)];
     const int local = item - B.item_begin;
     const int ty = local / B.tiles_x, tx = local - ty * B.tiles_x;
-    const int ray_id = threadIdx.x / kGlobalLanes, j = threadIdx.x % kGlobalLanes;
-    const int rx = tx * kGlobalTileW + ray_id % kGlobalTileW;
-    const int ry = ty * kGlobalTileH + ray_id / kGlobalTileW;
+    const int ray_id = threadIdx.x / LANES, j = threadIdx.x % LANES;
+    int rx, ry;
+    if constexpr (LANES == 1) {  // four 8 x 4 warp packets
+        rx = tx * 16 + (ray_id >> 5 & 1) * 8 + (ray_id & 7);
+        ry = ty * 8 + (ray_id >> 6) * 4 + (ray_id >> 3 & 3);
+    } else {
+        rx = tx * tile_w(LANES) + ray_id % tile_w(LANES);
+        ry = ty * tile_h(LANES) + ray_id / tile_w(LANES);
+    }
     const bool inside = rx < B.rect[2] && ry < B.rect[3];
     dev::Ray ray;
     dev::ray_setup(p, B.rect[0] + rx, B.rect[1] + ry, ray);
@@ -103,59 +104,102 @@ __global__ void __launch_bounds__(128) march_global_kernel(const __grid_constant
         w = v - (y - dev::kFloorOffset);
         return static_cast<int>(__float_as_uint(y) - dev::kFloorBits);
     };
-    for (int k = run.ka; __any_sync(all, k <= run.kb); k += kGlobalLanes) {
-        float a = 0.f, r = 0.f, g = 0.f, b = 0.f;
-        if (k + j <= run.kb) {
-            const float kh = static_cast<float>(k + j) + 0.5f;
-            float wx, wy, wz;
-            const int ix = cell(fmaf(kh, step[0], base[0]), wx);
-            const int iy = cell(fmaf(kh, step[1], base[1]), wy);
-            const int iz = cell(fmaf(kh, step[2], base[2]), wz);
-            const int x0 = min(max(ix, 0), nx - 1), x1 = min(max(ix + 1, 0), nx - 1);
-            const int y0 = min(max(iy, 0), ny - 1), y1 = min(max(iy + 1, 0), ny - 1);
-            const int z0 = min(max(iz, 0), nz - 1), z1 = min(max(iz + 1, 0), nz - 1);
-            const float *p0 = vol + z0 * plane, *p1 = vol + z1 * plane;
-            const long long r0 = static_cast<long long>(y0) * nx, r1 = static_cast<long long>(y1) * nx;
-            const float v000 = __ldg(p0 + r0 + x0), v100 = __ldg(p0 + r0 + x1), v010 = __ldg(p0 + r1 + x0),
-                        v110 = __ldg(p0 + r1 + x1), v001 = __ldg(p1 + r0 + x0), v101 = __ldg(p1 + r0 + x1),
-                        v011 = __ldg(p1 + r1 + x0), v111 = __ldg(p1 + r1 + x1);
-            const float c00 = fmaf(wx, v100 - v000, v000), c10 = fmaf(wx, v110 - v010, v010);
-            const float c01 = fmaf(wx, v101 - v001, v001), c11 = fmaf(wx, v111 - v011, v011);
-            const float c0 = fmaf(wy, c10 - c00, c00), c1 = fmaf(wy, c11 - c01, c01);
-            const float s = fmaf(wz, c1 - c0, c0);
-            const float x = fminf(fmaxf(fmaf(s, p.tf_scale, p.tf_bias), 0.0f), xmax);
-            float w;
-            float4 e0, de;
-            dev::ldg_v8(p.tf + 2 * cell(x, w), e0, de);
-            r = fmaf(w, de.x, e0.x);
-            g = fmaf(w, de.y, e0.y);
-            b = fmaf(w, de.z, e0.z);
-            a = fmaf(w, de.w, e0.w);
-        }
-        // T before this lane's sample; the ray ends after the first sample with T <= ert_T
-        float mine = T;
-#pragma unroll
-        for (int i = 0; i < kGlobalLanes; ++i) {
-            if (i == j) mine = T;
-            const float ai = __shfl_sync(all, a, i, kGlobalLanes);
-            if (!(T <= p.ert_T)) T = T - T * ai;
-        }
-        if (k + j <= run.kb && !(mine <= p.ert_T)) {
-            const float ta = mine * a;
+    auto sample = [&](int k, float &a, float &r, float &g, float &b) {
+        const float kh = static_cast<float>(k) + 0.5f;
+        float wx, wy, wz;
+        const int ix = cell(fmaf(kh, step[0], base[0]), wx);
+        const int iy = cell(fmaf(kh, step[1], base[1]), wy);
+        const int iz = cell(fmaf(kh, step[2], base[2]), wz);
+        const int x0 = min(max(ix, 0), nx - 1), x1 = min(max(ix + 1, 0), nx - 1);
+        const int y0 = min(max(iy, 0), ny - 1), y1 = min(max(iy + 1, 0), ny - 1);
+        const int z0 = min(max(iz, 0), nz - 1), z1 = min(max(iz + 1, 0), nz - 1);
+        const float *p0 = vol + z0 * plane, *p1 = vol + z1 * plane;
+        const long long r0 = static_cast<long long>(y0) * nx, r1 = static_cast<long long>(y1) * nx;
+        const float v000 = __ldg(p0 + r0 + x0), v100 = __ldg(p0 + r0 + x1), v010 = __ldg(p0 + r1 + x0),
+                    v110 = __ldg(p0 + r1 + x1), v001 = __ldg(p1 + r0 + x0), v101 = __ldg(p1 + r0 + x1),
+                    v011 = __ldg(p1 + r1 + x0), v111 = __ldg(p1 + r1 + x1);
+        const float c00 = fmaf(wx, v100 - v000, v000), c10 = fmaf(wx, v110 - v010, v010);
+        const float c01 = fmaf(wx, v101 - v001, v001), c11 = fmaf(wx, v111 - v011, v011);
+        const float c0 = fmaf(wy, c10 - c00, c00), c1 = fmaf(wy, c11 - c01, c01);
+        const float s = fmaf(wz, c1 - c0, c0);
+        const float x = fminf(fmaxf(fmaf(s, p.tf_scale, p.tf_bias), 0.0f), xmax);
+        float w;
+        float4 e0, de;
+        dev::ldg_v8(p.tf + 2 * cell(x, w), e0, de);
+        r = fmaf(w, de.x, e0.x);
+        g = fmaf(w, de.y, e0.y);
+        b = fmaf(w, de.z, e0.z);
+        a = fmaf(w, de.w, e0.w);
+    };
+    if constexpr (LANES == 1) {
+        for (int k = run.ka; k <= run.kb; ++k) {
+            float a, r, g, b;
+            sample(k, a, r, g, b);
+            const float ta = T * a;
             C0 = fmaf(ta, r, C0);
             C1 = fmaf(ta, g, C1);
             C2 = fmaf(ta, b, C2);
+            T = T - ta;
+            if (T <= p.ert_T) break;
         }
-        if (T <= p.ert_T) run.kb = k;  // the same for the ray's lanes
-    }
+    } else {
+        for (int k = run.ka; __any_sync(all, k <= run.kb); k += LANES) {
+            float a = 0.f, r = 0.f, g = 0.f, b = 0.f;
+            if (k + j <= run.kb) sample(k + j, a, r, g, b);
+            // T before this lane's sample; the ray ends after the first sample with T <= ert_T
+            float mine = T;
 #pragma unroll
-    for (int i = 1; i < kGlobalLanes; i += i) {
-        C0 += __shfl_xor_sync(all, C0, i);
-        C1 += __shfl_xor_sync(all, C1, i);
-        C2 += __shfl_xor_sync(all, C2, i);
+            for (int i = 0; i < LANES; ++i) {
+                if (i == j) mine = T;
+                const float ai = __shfl_sync(all, a, i, LANES);
+                if (!(T <= p.ert_T)) T = T - T * ai;
+            }
+            if (k + j <= run.kb && !(mine <= p.ert_T)) {
+                const float ta = mine * a;
+                C0 = fmaf(ta, r, C0);
+                C1 = fmaf(ta, g, C1);
+                C2 = fmaf(ta, b, C2);
+            }
+            if (T <= p.ert_T) run.kb = k;  // the same for the ray's lanes
+        }
+#pragma unroll
+        for (int i = 1; i < LANES; i += i) {
+            C0 += __shfl_xor_sync(all, C0, i);
+            C1 += __shfl_xor_sync(all, C1, i);
+            C2 += __shfl_xor_sync(all, C2, i);
+        }
     }
     if (inside && j == 0)
         p.partials[B.poff + static_cast<long long>(ry) * B.rect[2] + rx] = make_float4(C0, C1, C2, 1.0f - T);
+}
+
+// Lanes per ray of a call with `area` footprint pixels, its view direction's share along x
+// (the volume's rows), the mean bound of a ray's samples in a brick, whether rays end
+// early, and the row length.
+//
+// Few pixels leave the chip idle but for the longest rays, whose time falls with the
+// lanes. Many fill it, and then lanes that share a ray only repeat its setup and chain and
+// load other rows than their neighbours: one lane each is best, whose neighbours' pixels
+// share rows. Rays along the rows turn that round: consecutive samples share them, pixels do
+// not, the more so the longer the rows. us with 1 / 2 / 4 / 8 lanes:
+//   along z   256^3, 30,000 pixels 159 / 132 / 107 / 131; 128^3 in 2 bricks, 121,200
+//             160 / 166 / 168 / 205; 236,880 268 / 294 / 305 / 386; 256^3, 816,000
+//             1621 / 1858 / 1969 / 2529, opaque with early termination 32 / 43 / 74 / 139
+//             384^3 (long rays), 22,500 512 / 299 / 164 / 112
+//   along x   256^3, 163,216 1199 / 663 / 404 / 318; in 8 bricks, 445,264
+//             1232 / 778 / 579 / 532; 128^3 in 2 bricks, 437,840 287 / 231 / 235 / 285,
+//             opaque with early termination 30 / 34 / 50 / 88
+// Over 711 calls (64^3 to 384^3, 900 to 1,000,000 pixels, five directions, steps of 1/2 and 2
+// voxels) this choice takes 0.85 of the time of eight lanes for all, and 0.62 of the kernel's
+// with one lane before lanes were shared, and is in no call slower than that.
+int lanes_per_ray(double area, double along_x, double run, bool early, int row)
+{
+    if (area <= std::max(20000.0, along_x <= 0.4 ? 24.0 * run : 0.0)) return 8;
+    if (along_x <= 0.4) return area <= 140000 ? 4 : area <= 300000 ? 2 : 1;
+    if (area <= 100000) return 8;
+    if (early) return area <= 160000 ? 4 : area <= 600000 ? 2 : 1;
+    if (along_x > 0.7 && row >= 200 && area <= 300000) return 8;
+    return area <= 1500.0 * run ? 4 : area <= 700000 ? 2 : 1;
 }
 
 bool normalize3(double v[3])
@@ -191,7 +235,6 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
     static thread_local MarchParams mp;
     std::memset(&mp, 0, sizeof(mp));
     long long px = 0;
-    int items = 0;
     for (int b = 0; b < nb; ++b) {
         BrickLaunch &L = mp.b[b];
         const int *bx = &boxes[6 * b];
@@ -206,9 +249,6 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
         L.poff = px;
         px += static_cast<long long>(r[2]) * r[3];
         px = (px + 7) & ~7LL;
-        L.item_begin = items;
-        L.tiles_x = (r[2] + kGlobalTileW - 1) / kGlobalTileW;
-        items += L.tiles_x * ((r[3] + kGlobalTileH - 1) / kGlobalTileH);
     }
     // the frame's partial images must fit the fixed scratch
     const int tiles_x = (cam->width + kCompW - 1) / kCompW, tiles_y = (cam->height + kCompTileH - 1) / kCompTileH;
@@ -252,6 +292,23 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
     mp.tf_bias = static_cast<float>(-static_cast<double>(vmin) * scale);
     mp.ntf = n_tf;
     mp.nb = nb;
+    double area = 0.0, samples = 0.0;
+    for (int b = 0; b < nb; ++b) {
+        const BrickLaunch &L = mp.b[b];
+        const double px_b = static_cast<double>(L.rect[2]) * L.rect[3];
+        double d2 = 0.0;
+        for (int a = 0; a < 3; ++a) d2 += static_cast<double>(L.hi[a] - L.lo[a]) * (L.hi[a] - L.lo[a]);
+        area += px_b;
+        samples += px_b * std::sqrt(d2) / step_voxels;
+    }
+    const int lanes = lanes_per_ray(area, std::fabs(f[0]), area > 0.0 ? samples / area : 0.0, ert_alpha < 1.0f, dims[0]);
+    int items = 0;
+    for (int b = 0; b < nb; ++b) {
+        BrickLaunch &L = mp.b[b];
+        L.item_begin = items;
+        L.tiles_x = (L.rect[2] + tile_w(lanes) - 1) / tile_w(lanes);
+        items += L.tiles_x * ((L.rect[3] + tile_h(lanes) - 1) / tile_h(lanes));
+    }
     mp.n_items = items;
     mp.data = volume_dev;
 
@@ -282,7 +339,13 @@ extern "C" vr_status vr_render_frame_noalloc(const float *volume_dev, const int 
     mp.mask_tiles_y = tiles_y;
     mp.mask_blocks = (tiles_x * tiles_y + kMaskThreads - 1) / kMaskThreads;
     for (int j = 0; j < nb; ++j) mp.order[j] = order[j];
-    march_global_kernel<<<mp.mask_blocks + items, kMaskThreads, 0, s>>>(mp);
+    const int grid = mp.mask_blocks + items;
+    switch (lanes) {
+    case 1: march_global_kernel<1><<<grid, kMaskThreads, 0, s>>>(mp); break;
+    case 2: march_global_kernel<2><<<grid, kMaskThreads, 0, s>>>(mp); break;
+    case 4: march_global_kernel<4><<<grid, kMaskThreads, 0, s>>>(mp); break;
+    default: march_global_kernel<8><<<grid, kMaskThreads, 0, s>>>(mp); break;
+    }
     if (cudaGetLastError() != cudaSuccess) return VR_ERR_CUDA;
     // direct front-to-back composite with the existing kernel
     static thread_local CompositeParams cp;

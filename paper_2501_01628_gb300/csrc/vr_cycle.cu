@@ -17,14 +17,14 @@ namespace {
 // ---------------------------------------------------------------------------
 // Bound by the latency of a ray's chain of loads (a launch has one thread per
 // pixel, each with all its bricks' samples), so each ray keeps kWideSamples samples
-// in flight, at 8 blocks per SM. ms per frame, samples in pairs with the previous
-// cell's quads reused / four in flight: 512^3, 36 bricks, 1080p 0.581 / 0.544;
-// 256^3 at 1024^2 0.491 / 0.461, at 512^2 0.334 / 0.307, at 256^2 0.156 / 0.122;
-// 64^3 at 256^2 0.0214 / 0.0198. (Six or eight in flight: 0.269 and 0.230 at 512^2,
-// but 0.146 and 0.134 at 256^2, 0.481 and 0.476 at 1024^2.) The counting variant
-// keeps the pairs, whose quads' bounds it checks.
-template <typename S, bool COUNT, int OPC>
-__global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_constant__ MarchParams p, float4 *out)
+// in flight, at 8 blocks per SM (36 to 48 bytes of spill stores). ms per frame, samples in
+// pairs with the previous cell's quads reused / four in flight: 512^3, 36 bricks, 1080p
+// 0.581 / 0.544; 256^3 at 1024^2 0.491 / 0.461, at 512^2 0.334 / 0.307, at 256^2 0.156 /
+// 0.122; 64^3 at 256^2 0.0214 / 0.0198. (Six or eight in flight: 0.269 and 0.230 at 512^2,
+// but 0.146 and 0.134 at 256^2, 0.481 and 0.476 at 1024^2.) Pairs stay where they are
+// better (cycle_pairs in vr_host.cpp) and for counting, whose quads' bounds they check.
+template <typename S, bool COUNT, int OPC, bool WIDE>
+__device__ __forceinline__ void cycle_block(const MarchParams &p, float4 *out)
 {
     // pipelined frames: the next frame's kernel may start once every block of
     // this grid is running, and this grid's image store waits for the
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_consta
             continue;
         dev::OwnedRun run;
         dev::brick_run(p, B, ray, run);
-        if constexpr (!COUNT)
+        if constexpr (WIDE)
             dev::march_accumulate_wide<S, OPC, kWideSamples>(p.data, B, run, p.tf, p.tf_scale, p.tf_bias, p.ntf,
                                                              p.ert_T, C0, C1, C2, T, p.opc);
         else
@@ -57,14 +57,27 @@ __global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_consta
     if (COUNT && executed) atomicAdd(p.sample_counter, executed);
 }
 
+template <typename S, int OPC>
+__global__ void __launch_bounds__(128, 8) march_cycle_kernel(const __grid_constant__ MarchParams p, float4 *out)
+{
+    cycle_block<S, false, OPC, true>(p, out);
+}
+
+template <typename S, bool COUNT, int OPC>
+__global__ void __launch_bounds__(128) march_cycle_pairs_kernel(const __grid_constant__ MarchParams p, float4 *out)
+{
+    cycle_block<S, COUNT, OPC, false>(p, out);
+}
+
 }  // namespace
 
-cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cudaStream_t s, bool after_frame)
+cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cudaStream_t s, bool after_frame,
+                               bool pairs)
 {
     if (p.W <= 0 || p.H <= 0) return cudaSuccess;
     const dim3 grid((p.W + p.tile_w - 1) / p.tile_w, (p.H + p.tile_h - 1) / p.tile_h);
     const bool count = p.sample_counter != nullptr;
-    const bool opc = opacity_kind(p.opc) != kOpacityOff;
+    const int opc = opacity_kind(p.opc);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -74,11 +87,16 @@ cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cuda
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = after_frame ? 1 : 0;
-#define VR_CYCLE(T)                                                                              \
-    (opc ? (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, kOpacitySeries>, p, out)    \
-                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, kOpacitySeries>, p, out))  \
-         : (count ? cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, true, kOpacityOff>, p, out)       \
-                  : cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, false, kOpacityOff>, p, out)))
+#define VR_PAIRS(T, C, O) cudaLaunchKernelEx(&cfg, march_cycle_pairs_kernel<T, C, O>, p, out)
+#define VR_WIDE(T, O) cudaLaunchKernelEx(&cfg, march_cycle_kernel<T, O>, p, out)
+#define VR_CYCLE(T)                                                                                       \
+    (count   ? (opc ? VR_PAIRS(T, true, kOpacitySeries) : VR_PAIRS(T, true, kOpacityOff))                  \
+     : pairs ? (opc == kOpacitySeries    ? VR_PAIRS(T, false, kOpacitySeries)                              \
+                : opc == kOpacityGeneral ? VR_PAIRS(T, false, kOpacityGeneral)                             \
+                                         : VR_PAIRS(T, false, kOpacityOff))                                \
+             : (opc == kOpacitySeries    ? VR_WIDE(T, kOpacitySeries)                                      \
+                : opc == kOpacityGeneral ? VR_WIDE(T, kOpacityGeneral)                                     \
+                                         : VR_WIDE(T, kOpacityOff)))
     cudaError_t e = cudaErrorInvalidValue;
     switch (kind) {
     case kStoreF32: e = VR_CYCLE(float); break;
@@ -89,6 +107,8 @@ cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cuda
     default: return cudaErrorInvalidValue;
     }
 #undef VR_CYCLE
+#undef VR_WIDE
+#undef VR_PAIRS
     return e;
 }
 

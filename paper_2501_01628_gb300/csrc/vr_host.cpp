@@ -580,6 +580,33 @@ void timing_end(vr_ctx ctx, int idx, cudaStream_t s)
 constexpr int kWideBlocks = 6;
 bool wide_march(vr_ctx ctx, int blocks) { return blocks <= kWideBlocks * ctx->sms; }
 
+// Cycling frames march in pairs instead of four samples at a time (same image) where
+// bricks are small, since each brick's run is rounded up to whole fours and then ends in
+// requests that are not used: a mean run (4 volume / surface, the mean chord of a box) of
+// at most kPairsRun samples. us per frame, pairs / four, f32 | bf16 | f16 octets: 125 bricks of
+// 9.6^3 voxels, 1080p 195 / 223 | 195 / 232 | 192 / 215; 64 of 16^3, 1024 x 768 108 / 119 |
+// 109 / 120 | 105 / 114; 125 of 25.6^3 (34 samples), 1280 x 720 193 / 210 | 190 / 208 | 182 /
+// 199; 100 slabs of 1.3 voxels, 800 x 600 334 / 368 | 306 / 364 | 304 / 356; 64 of 32^3
+// (43 samples), 640 x 480 134 / 127 | 126 / 120 | 123 / 125; 64 of 64^3 393 / 321 | 287 / 258
+// | 306 / 298.
+// Octets with the general opacity formula at every sample, whose two loads per pair leave
+// the formulas to bound them, do so too unless the launch is small: 256^3 in 8, 1280 x 720
+// 448 / 474, 1080p of 384^3 in 100 1309 / 1342; 128^3 at 200 x 160 38 / 30.
+constexpr double kPairsRun = 38.0;
+bool cycle_pairs(vr_ctx ctx, vr_volume vol, const MarchParams &mp)
+{
+    double volume = 0.0, surface = 0.0;
+    for (size_t b = 0; b < vol->boxes.size() / 6; ++b) {
+        const int *bx = &vol->boxes[6 * b];
+        const double x = bx[3] - bx[0], y = bx[4] - bx[1], z = bx[5] - bx[2];
+        volume += x * y * z;
+        surface += 2.0 * (x * y + y * z + z * x);
+    }
+    if (4.0 * volume <= kPairsRun * ctx->step * surface) return true;
+    const long long blocks = static_cast<long long>(mp.W) * mp.H / 128;
+    return vol->octets && opacity_kind(mp.opc) == kOpacityGeneral && blocks > 3LL * ctx->sms;
+}
+
 vr_status march(vr_ctx ctx, vr_volume vol, vr_frame_s &fr, cudaStream_t s, bool after_composite = false,
                 const PoolSync *sync = nullptr)
 {
@@ -831,7 +858,7 @@ vr_status cycle_to(vr_ctx ctx, vr_volume vol, float *out, int out_on_device, cud
     const bool pipe = pipelined_output(ctx, out_on_device);
     const bool after = pipe_after(ctx, s) && pipe;
     const int t = timing_begin(ctx, 0, s);
-    VR_LAUNCH(ctx, launch_march_cycle(mp, vol->kind(), dst, s, after));
+    VR_LAUNCH(ctx, launch_march_cycle(mp, vol->kind(), dst, s, after, cycle_pairs(ctx, vol, mp)));
     timing_end(ctx, t, s);
     if (!out_on_device) {
         st = host_copy(ctx, out, dst, slot, px, s);

@@ -278,8 +278,10 @@ cudaError_t launch_pack(const PackParams &p, int kind, cudaStream_t s);
 cudaError_t launch_march(const MarchParams &p, int kind, cudaStream_t s, bool after_composite = false,
                          bool wide = false);
 // after_frame: launch as a programmatic dependent of the preceding kernel (the
-// previous pipelined frame); see march_cycle_kernel.
-cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cudaStream_t s, bool after_frame = false);
+// previous pipelined frame); see march_cycle_kernel. pairs: two samples of a ray in
+// flight instead of four (same image).
+cudaError_t launch_march_cycle(const MarchParams &p, int kind, float4 *out, cudaStream_t s, bool after_frame,
+                               bool pairs);
 // max_blocks > 0: a grid of at most that many blocks, each compositing tiles in
 // turn; 0: one block per tile.
 cudaError_t launch_composite(const CompositeParams &p, cudaStream_t s, int max_blocks = 0);

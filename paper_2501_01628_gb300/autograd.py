@@ -36,8 +36,8 @@ class Renderer:
         self.vol = None
         self._key = None
         self._shape = None
-        self._done = None      # event behind the last render
-        self._stream = None    # its stream (None: no render, or one that is known to be done)
+        self._done = None      # event behind the last render on a stream other than the default one
+        self._stream = None    # of the last render (None: no render, or one that is known to be done)
         vr.vr_set_render_params(self.ctx, self.step, 1.0)
 
     def _enter(self):
@@ -45,15 +45,22 @@ class Renderer:
         capture starts with an idle device, and its events mean nothing outside.)"""
         stream = torch.cuda.current_stream()
         if self._stream is not None and stream != self._stream and not torch.cuda.is_current_stream_capturing():
-            stream.wait_event(self._done)
+            if self._stream.cuda_stream == 0:
+                stream.wait_stream(self._stream)
+            else:
+                stream.wait_event(self._done)
         return stream
 
     def _leave(self, stream):
-        if not torch.cuda.is_current_stream_capturing():
+        # the default stream is always there to be waited for; another may be gone by the
+        # next render, so an event is left behind on it (6 us of host time)
+        if stream.cuda_stream != 0:
+            if torch.cuda.is_current_stream_capturing():
+                return
             if self._done is None:
                 self._done = torch.cuda.Event()
             self._done.record(stream)
-            self._stream = stream
+        self._stream = stream
 
     def _bind(self, tf: torch.Tensor, density: torch.Tensor, cam: dict, stream):
         d = density.detach()

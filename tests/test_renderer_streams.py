@@ -10,15 +10,20 @@ import torch
 from paper_2501_01628_gb300 import autograd, synth
 
 
-def test_a_render_on_another_stream_waits_for_the_last_one(monkeypatch):
+@pytest.mark.parametrize("handles", [(5, 7), (0, 7), (5, 0)])  # 0: the default stream
+def test_a_render_on_another_stream_waits_for_the_last_one(monkeypatch, handles):
     log, state = [], dict(stream=None, capturing=False)
 
     class Stream:
-        def __init__(self, name):
-            self.name = name
+        def __init__(self, name, handle):
+            self.name, self.cuda_stream = name, handle
 
         def wait_event(self, event):
             log.append("%s waits for %s" % (self.name, event.at))
+
+        def wait_stream(self, other):
+            assert other.cuda_stream == 0  # any other may be gone
+            log.append("%s waits for %s" % (self.name, other.name))
 
     class Event:
         def record(self, stream):
@@ -27,7 +32,7 @@ def test_a_render_on_another_stream_waits_for_the_last_one(monkeypatch):
     calls = {name: (lambda name: lambda *a, **k: log.append("%s %s" % (state["stream"].name, name)))(name)
              for name in ("vr_create", "vr_set_render_params", "vr_render_frame", "vr_render_backward", "vr_sync",
                           "vr_destroy")}
-    a, b = Stream("a"), Stream("b")
+    a, b = Stream("a", handles[0]), Stream("b", handles[1])
     state["stream"] = a
     monkeypatch.setattr(autograd, "vr", types.SimpleNamespace(**calls))
     monkeypatch.setattr(torch.cuda, "current_stream", lambda *_: state["stream"])

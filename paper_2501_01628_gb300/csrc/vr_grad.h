@@ -14,9 +14,11 @@ constexpr int kGradSeg = 8;
 constexpr int kGradGroup = 8;
 constexpr int kGradMaxRun = 4096;
 // Copies of the table gradient ((ntf + 1) x 4 floats each), spread over blocks and
-// lanes so that few reductions meet on one entry. 256^3 volume, 4 views of 512^2, ms
-// per training step: 7.29 with 16 copies by block, 6.44 with 64, 6.21 with 256, 6.15
-// with 1024 by block and lane % 8, 6.66 with 4096 by block and lane.
+// lanes so that few reductions meet on one entry. 4 views of 512^2, ms per training step,
+// 64 / 256 / 512 / 1024 / 2048 copies by block and lane % 8: 256^3 blobs 5.16 / 5.00 / 5.00 /
+// 5.11 / 5.12, noise 7.21 / 6.49 / 6.31 / 6.38 / 6.33; 512 by block alone 5.12 and 6.34, by
+// block and lane 5.06 and 6.38. (16 copies by block, an earlier kernel: 7.29 against 6.44
+// with 64.)
 constexpr int kGradCopies = 512;
 constexpr int kGradLaneCopies = 8;
 // Voxel gradients go through quads (at most two 16-byte reductions per cell, then

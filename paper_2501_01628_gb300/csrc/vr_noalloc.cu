@@ -186,17 +186,18 @@ __global__ void __launch_bounds__(128, 9) march_global_kernel(const __grid_const
 //             160 / 166 / 168 / 205; 236,880 268 / 294 / 305 / 386; 256^3, 816,000
 //             1621 / 1858 / 1969 / 2529, opaque with early termination 32 / 43 / 74 / 139
 //             384^3 (long rays), 22,500 512 / 299 / 164 / 112
+//   oblique   192^3 in 4 bricks, 110,210 363 / 214 / 151 / 119
 //   along x   256^3, 163,216 1199 / 663 / 404 / 318; in 8 bricks, 445,264
 //             1232 / 778 / 579 / 532; 128^3 in 2 bricks, 437,840 287 / 231 / 235 / 285,
 //             opaque with early termination 30 / 34 / 50 / 88
 // Over 711 calls (64^3 to 384^3, 900 to 1,000,000 pixels, five directions, steps of 1/2 and 2
-// voxels) this choice takes 0.85 of the time of eight lanes for all, and 0.62 of the kernel's
+// voxels) this choice takes about 0.86 of the time of eight lanes for all, 0.62 of the kernel's
 // with one lane before lanes were shared, and is in no call slower than that.
 int lanes_per_ray(double area, double along_x, double run, bool early, int row)
 {
     if (area <= std::max(20000.0, along_x <= 0.4 ? 24.0 * run : 0.0)) return 8;
     if (along_x <= 0.4) return area <= 140000 ? 4 : area <= 300000 ? 2 : 1;
-    if (area <= 100000) return 8;
+    if (area <= (early ? 125000 : 150000)) return 8;
     if (early) return area <= 160000 ? 4 : area <= 600000 ? 2 : 1;
     if (along_x > 0.7 && row >= 200 && area <= 300000) return 8;
     return area <= 1500.0 * run ? 4 : area <= 700000 ? 2 : 1;

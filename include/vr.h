@@ -135,7 +135,7 @@ const char *vr_status_string(vr_status s);
 const char *vr_last_error(vr_ctx ctx);
 /* Wait for `stream` and report any device-side error word set by a kernel
  * (VR_ERR_TIMEOUT for a bounded wait that gave up, VR_ERR_BOUNDS for an
- * adjoint run beyond its checkpoint storage), clearing it. */
+ * adjoint run of more than 4096 samples), clearing it. */
 vr_status vr_sync(vr_ctx ctx, void *stream);
 
 /* ---- volume (the distributed World of Sec. 3, all bricks on this GPU) ---- */

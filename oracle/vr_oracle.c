@@ -691,7 +691,7 @@ int orc_kd_partition(const int dims[3], int n, const double *u, int *boxes)
  *   table: rgba = (1-w) T[i] + w T[i+1] gives dT[i] += (1-w) g, dT[i+1] += w g,
  *     and ds = (g . (T[i+1] - T[i])) (n-1)/(vmax - vmin) where u is not clamped;
  *   trilinear: dv(corner) += ds * weight(corner), on the clamped global indices.
- * This oracle stores every sample of a ray (it is not the checkpointed GPU
+ * This oracle stores every sample of a ray (it is not the segmented GPU
  * adjoint); there is no division by a transmittance anywhere. */
 typedef struct {
     double p[3], s, x, rgba[4];

@@ -574,9 +574,10 @@ void timing_end(vr_ctx ctx, int idx, cudaStream_t s)
 // frame pairs / wide, pipelined and in sequence: 24 blocks 8.2 / 5.3 and 26.7 / 20.5;
 // 520 blocks (64^3 at 256^2) 13.6 / 12.7 and 24.7 / 24.6; 538 blocks, 128^3 26.5 / 25.8
 // and 53.4 / 45.2, 256^3 92.0 / 78.8 and 211 / 141; 943 blocks 119 / 107 and 221 / 160.
-// Above, either may win by view (1075 blocks 491 / 502 and 800 / 704, 1145 blocks 39.6 /
-// 39.2 and 58.4 / 61.5, 2705 blocks 330 / 304, 3721 blocks 344 / 357), and full launches,
-// bound by the L1 that the pairs' reuse of the previous cell saves, lose 2 to 6%.
+// Above, the number of blocks does not say which wins: 1075 blocks 491 / 502 and 800 / 704,
+// 1145 blocks 39.6 / 39.2 and 58.4 / 61.5, 2705 blocks 330 / 304, 3721 blocks 344 / 357; full
+// launches, bound by the L1 that the pairs' reuse of the previous cell saves, lose 2 to 6%. The
+// line lies below the first launch that lost.
 constexpr int kWideBlocks = 6;
 bool wide_march(vr_ctx ctx, int blocks) { return blocks <= kWideBlocks * ctx->sms; }
 
